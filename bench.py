@@ -60,7 +60,7 @@ WORKLOADS = {
 
 
 # Sources the panel kernel is built from (kernel, plan, fixed-point helpers, shared structures).
-PANEL_SOURCES = ("dq_panel.cu", "dq_panel.cpp", "dq_fixed.cuh", "dq_internal.h")
+PANEL_SOURCES = ("dq_panel.cu", "dq_panel.cuh", "dq_panel.cpp", "dq_fixed.cuh", "dq_internal.h")
 
 
 def kernel_source_hash() -> str:

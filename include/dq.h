@@ -179,7 +179,9 @@ int dq_make_terms(const dq_sector* s, const dq_term* terms, int n_terms, dq_term
  * (Nbits * L_1 <= 14) and P_0 of at most 24, no n_i n_j pair terms, D < 2^40, at most 31 hop
  * bonds and 4096 hop amplitude entries (bonds x Q x Q), 64 P_0 and cut hops per panel; any
  * coefficient per hop bond and any site function (the per-term form's integer coefficients, so
- * it gives the general kernel's y). */
+ * it gives the general kernel's y). With three or more subsystems the value names the form that fits
+ * the sector's own partition; sectors of at least 2^19 rows whose operator fits two halves of the
+ * lattice run the panel kernel on those halves instead, with the same y. */
 int dq_terms_path(const dq_terms* t, int* path);
 
 /* Compile terms in the cluster-merged form of App. C instead: the terms are grouped into clusters

@@ -163,6 +163,12 @@ struct PanelPlan {
     // three or more subsystems (the warp-panel kernel): prefix bits of the Sz Sz bonds across the
     // cut, per class and per position b of P_1 (the per-panel counters are built on the device)
     uint32_t xzA[kPanelMaxK][32];
+    // split order (dq_panel.cpp): canonical index of a row = piece[panel * npiece + (rowy >> 16)] +
+    // (rowy & 0xffff), rowy per P_1 pattern as in t1states; NULL when panels are canonical ranges
+    int Llow, npiece;
+    uint32_t lowfirst[16];        // per particle number: first pattern of the Llow low bits
+    const uint32_t* rowy;
+    uint64_t* piece;
 };
 
 // What the warp-panel kernel needs of the sector to rank a prefix pattern on the device: Eq.
@@ -301,6 +307,7 @@ struct dq_terms {
     std::vector<void*> dev_allocs;
     int max_hops;  // upper bound on off-diagonal elements per row
     bool panel_ok = false;     // the panel product applies (see PanelPlan)
+    bool split = false;        // the panel kernel runs on the split order (three or more subsystems)
     bool pb_ok = false;        // the per-bond panel product applies (PanelPB)
     bool pw_ok = false;        // the warp-panel product applies (three or more subsystems, PanelPlan)
     bool pq_ok = false;        // the boson panel product applies (Q > 2, PanelQ)
@@ -364,6 +371,7 @@ int launch_panel_q_ws(const dq_sector* s, const dq_terms* t, const void* x, void
                       void* stream);
 int launch_panel_w_ws(const dq_sector* s, const dq_terms* t, const void* x, void* y, int dtype, void* ws,
                       void* stream);
+int launch_panel_pieces(const dq_sector* s, const PanelPlan& P);
 size_t panel_scratch_bytes(const dq_sector* s, int dtype);
 int launch_panel_matvec_ws(const dq_sector* s, const dq_terms* t, const void* x, void* y, int dtype, void* scratch,
                            void* stream);

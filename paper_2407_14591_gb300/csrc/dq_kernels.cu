@@ -442,7 +442,7 @@ static int launch_matvec_f32x(const dq_sector* s, dq_terms* t, const float* x, f
 int launch_matvec(const dq_sector* s, const dq_terms* t, const void* x, void* y, int dtype, int nrhs, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     if (t->cluster) return launch_cluster_matvec(s, const_cast<dq_terms*>(t), x, y, dtype, nrhs, stream);
-    if (t->panel_ok && nrhs == 1) return launch_panel_matvec(s, const_cast<dq_terms*>(t), x, y, dtype, stream);
+    if ((t->panel_ok || t->split) && nrhs == 1) return launch_panel_matvec(s, const_cast<dq_terms*>(t), x, y, dtype, stream);
     if (t->pw_ok && nrhs == 1) return launch_panel_w(s, const_cast<dq_terms*>(t), x, y, dtype, stream);
     if (t->pq_ok && nrhs == 1) return launch_panel_q(s, const_cast<dq_terms*>(t), x, y, dtype, stream);
     if (t->pb_ok && nrhs == 1) return launch_panel_pb(s, const_cast<dq_terms*>(t), x, y, dtype, stream);

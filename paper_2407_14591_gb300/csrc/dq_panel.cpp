@@ -27,6 +27,16 @@
 // own two-subsystem canonical order (Eq. (index) restricted to the tail). That order depends on
 // the tail's particle number only; the host tabulates it (tail pattern -> local index) from the
 // sector's own rank and checks every panel's first and last row.
+//
+// Large sectors of three or more subsystems take neither: the panel kernel works on x in the order of
+// a split into TWO subsystems of its own (the "split order": P_0 = the upper L - L_1 sites, P_1 the
+// lower L_1 <= 15), whatever the sector's partition is. The prepass that makes the fixed-point copy of
+// x gathers it into that order and the kernel's stores go back through the same map. A panel of the
+// split order is a few contiguous pieces of the canonical order: the suffix bits that lie in whole
+// subsystems (Llow of them) run through a contiguous range whose order depends on their particle
+// number only, one piece per pattern of the suffix bits above. One short panel per warp (k_panel_w),
+// or a tail of two short subsystems, reads about 50 partner panels per panel where 15 sites read 34.
+// 6 x 5 lattice, N = 15: three subsystems, FP32 21.4 -> 10.7 ms a product; five, FP64 23.5 -> 14.9 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -37,6 +47,8 @@
 #include "dq_internal.h"
 
 namespace dq {
+
+constexpr uint64_t kSplitMinDim = 1ull << 19;
 
 // Exponent of the lowest set bit of v's mantissa: v = m * 2^e with m odd.
 static int low_exponent(double v) {
@@ -116,21 +128,50 @@ static int build_panel_w(const dq_sector* s, PanelPlan& P, const std::vector<uin
     return DQ_OK;
 }
 
-int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
-                     const std::vector<std::pair<std::pair<int, int>, std::pair<double, double>>>& pairs, dq_terms* t) {
-    t->panel_ok = false;
-    t->pw_ok = false;
-    if (s->Q != 2 || s->n_sub < 2 || !uniform_lin || s->wide) return DQ_OK;
+// P_1 of the split order: the lower half of the sites, at most 15.
+static int split_sites(const dq_sector* s) { return std::min(15, s->L / 2); }
+
+// The split order pays for its gather of x and its scattered stores where its panels are longer than
+// those of the sector's own form (see build_panel_plan for tails of two subsystems): against warp
+// panels 1.1 to 1.6 times faster from 2 M rows on (chains of 24 to 28 sites, 4 x 6, 5 x 5 and 4 x 7
+// lattices), 2.0 times on the 6 x 5 lattice with three subsystems and FP32 vectors; against tails two
+// or more sites shorter 2.5 to 6 times, already at 0.7 M rows (22 sites, five subsystems: 0.266 ->
+// 0.059 ms). Smaller sectors keep their own form.
+static bool use_split_order(const dq_sector* s) {
+    const int L1 = split_sites(s);
+    return s->n_sub >= 3 && s->D >= kSplitMinDim && s->D < (1ull << 48) && L1 > 10 && s->L - L1 <= 16;
+}
+
+// Bits of the lowest whole subsystems inside a suffix of L1 bits (L1 itself when the suffix lies
+// inside the last subsystem, whose order is lexicographic).
+static int whole_bits(const dq_sector* s, int L1) {
+    if (L1 <= s->Lk[s->n_sub - 1]) return L1;
+    int low = 0;
+    for (int k = s->n_sub - 1; k >= 0 && low + s->Lk[k] <= L1; --k) low += s->Lk[k];
+    return low;
+}
+
+// One form of the plan: the sector's own order or the split order. *fits: the operator's bonds and
+// coefficients fit the form; with check_only nothing else is done.
+static int build_form(const dq_sector* s, double C,
+                      const std::vector<std::pair<std::pair<int, int>, std::pair<double, double>>>& pairs, dq_terms* t,
+                      bool split, bool check_only, bool* fits) {
+    *fits = false;
     // the warp-panel kernel for three or more subsystems, and for two when the panels are small
     // (P_1 of 8 to 10 sites: at most 252 rows, which leave most of a 1024-thread CTA idle)
     const int ns = s->n_sub;
     const bool warp = s->Lk[ns - 1] >= 8 && s->Lk[ns - 1] <= 10;
     const bool tail = ns >= 3 && !warp;  // P_1 = the last two subsystems
-    const int L1 = tail ? s->Lk[ns - 2] + s->Lk[ns - 1] : s->Lk[ns - 1], L0 = s->L - L1, N = s->N;
+    int L1 = tail ? s->Lk[ns - 2] + s->Lk[ns - 1] : s->Lk[ns - 1], L0 = s->L - L1;
+    const int N = s->N;
     if (warp) {
         if (ns > kPWMaxSub || L0 > 24) return DQ_OK;
     } else if (L1 > 15 || L1 < 1 || L0 > (tail ? 22 : 16)) {
         return DQ_OK;
+    }
+    if (split) {
+        L1 = split_sites(s);
+        L0 = s->L - L1;
     }
     PanelPlan& P = t->pp;
     std::memset(&P, 0, sizeof P);
@@ -273,9 +314,22 @@ int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
     for (int k = 0; k < P.nA; ++k)
         if (!scaled(Avals[k], P.MA[k])) return DQ_OK;
     P.emin = emin;
+    *fits = true;
+    if (check_only) return DQ_OK;
     // P_1 tables (local index within its particle-number sector, and the states per sector)
     std::vector<uint16_t> t1rank, t1states;
-    if (!tail) {
+    if (split) {  // lexicographic inside each particle number
+        t1rank.assign((size_t)1 << L1, 0);
+        for (int n = 0; n <= L1 + 1 && n < 18; ++n) {
+            P.t1start[n] = (uint32_t)t1states.size();
+            for (uint32_t w = 0; n <= L1 && w < (1u << L1); ++w)
+                if (__builtin_popcount(w) == n) {
+                    t1rank[w] = (uint16_t)(t1states.size() - P.t1start[n]);
+                    t1states.push_back((uint16_t)w);
+                }
+            P.t1len[n] = (uint32_t)t1states.size() - P.t1start[n];
+        }
+    } else if (!tail) {
         const int tl = s->dev.tab[ns - 1];
         const auto& rt = s->h.rank_tab[tl];
         const auto& ut = s->h.unrank_tab[tl];
@@ -324,13 +378,28 @@ int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
             at += P.t1len[n];
         }
     }
-    if (warp) return build_panel_w(s, P, t1rank, t1states, xz, t);
+    if (warp && !split) return build_panel_w(s, P, t1rank, t1states, xz, t);
     // panels in canonical order: particle number of P_0, then its local order
     std::vector<uint32_t> ps0;
     std::vector<uint64_t> pst;
     int cmax = 0;
-    std::vector<uint64_t> tail_start;  // first index of every prefix pattern's panel (tail form)
-    if (!tail) {
+    std::vector<uint64_t> tail_start;  // first index of every prefix pattern's panel (tail form, split order)
+    if (split) {
+        tail_start.assign((size_t)1 << L0, UINT64_MAX);
+        uint64_t at = 0;
+        for (int n0 = 0; n0 <= L0; ++n0) {
+            const int n1 = N - n0;
+            if (n1 < 0 || n1 > L1) continue;
+            for (uint32_t s0 = 0; s0 < (1u << L0); ++s0) {
+                if (__builtin_popcount(s0) != n0) continue;
+                tail_start[s0] = at;
+                ps0.push_back(s0);
+                pst.push_back(at);
+                at += P.t1len[n1];
+            }
+            cmax = std::max(cmax, (int)P.t1len[n1]);
+        }
+    } else if (!tail) {
         const auto& u0 = s->h.unrank_tab[s->dev.tab[0]];
         const auto& s0s = s->h.sec_start[s->dev.tab[0]];
         for (int n0 = 0; n0 <= L0; ++n0) {
@@ -364,7 +433,7 @@ int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
             pst.push_back(e.first);
         }
     }
-    auto start_of = [&](uint32_t p) -> uint64_t { return tail ? tail_start[p] : s->h.c0_tab[p]; };
+    auto start_of = [&](uint32_t p) -> uint64_t { return tail_start.empty() ? s->h.c0_tab[p] : tail_start[p]; };
     P.npanels = (uint32_t)ps0.size();
     P.cmax = cmax;
     // per-panel diagonal counters (see PanelDiag)
@@ -436,8 +505,64 @@ int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
     if ((rc = dev_upload(t->dev_allocs, pdiag.data(), pdiag.size() * sizeof(PanelDiag), &p))) return rc;
     P.diag = (const PanelDiag*)p;
     P.c0 = s->dev.c0_tab;
-    t->panel_ok = true;
+    if (split) {
+        // canonical order of the rows of a panel (see the file comment)
+        const int low = whole_bits(s, L1), L = s->L;
+        const uint32_t lowmask = (1u << low) - 1;
+        P.Llow = low;
+        P.npiece = 1 << (L1 - low);
+        std::vector<std::vector<uint32_t>> byn(low + 1);
+        for (uint32_t w = 0; w <= lowmask; ++w) byn[__builtin_popcount(w)].push_back(w);
+        std::vector<uint32_t> pos((size_t)lowmask + 1, 0), rowy(t1states.size());
+        for (int n = 0; n <= low; ++n) {
+            P.lowfirst[n] = byn[n][0];
+            const int up = N - n;
+            if (up < 0 || up > L - low) continue;  // no state of the sector has n particles there
+            const u128 rep = (((u128)1 << up) - 1) << low;
+            std::vector<std::pair<uint64_t, uint32_t>> r;
+            for (uint32_t w : byn[n]) r.push_back({host_rank(s, rep | w), w});
+            std::sort(r.begin(), r.end());
+            for (size_t q = 0; q < r.size(); ++q) {
+                if (r[q].first != r[0].first + q) return set_error(DQ_ERANGE, "split order: the suffix is not contiguous");
+                pos[r[q].second] = (uint32_t)q;
+            }
+            P.lowfirst[n] = r[0].second;
+        }
+        for (size_t q = 0; q < t1states.size(); ++q)
+            rowy[q] = pos[t1states[q] & lowmask] | ((uint32_t)(t1states[q] >> low) << 16);
+        if ((rc = dev_upload(t->dev_allocs, rowy.data(), rowy.size() * 4, &p))) return rc;
+        P.rowy = (const uint32_t*)p;
+        if ((rc = dev_upload(t->dev_allocs, nullptr, (size_t)P.npanels * P.npiece * 8, &p))) return rc;
+        P.piece = (uint64_t*)p;
+        if (int e = launch_panel_pieces(s, P))
+            return set_error(DQ_ECUDA, "panel pieces: %s", cudaGetErrorString((cudaError_t)e));
+    }
+    t->split = split;
+    (warp ? t->pw_ok : t->panel_ok) = true;
     return DQ_OK;
+}
+
+int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
+                     const std::vector<std::pair<std::pair<int, int>, std::pair<double, double>>>& pairs, dq_terms* t) {
+    t->panel_ok = false;
+    t->pw_ok = false;
+    t->split = false;
+    if (s->Q != 2 || s->n_sub < 2 || !uniform_lin || s->wide) return DQ_OK;
+    bool fits = false;
+    if (use_split_order(s)) {
+        // the form dq_terms_path reports is the sector's own, whichever kernel runs
+        bool own = false;
+        if (int rc = build_form(s, C, pairs, t, false, true, &own)) return rc;
+        const int ns = s->n_sub, last = s->Lk[ns - 1], tail = s->Lk[ns - 2] + last;
+        const bool long_tail = own && (last < 8 || last > 10) && tail >= split_sites(s) - 1;
+        if (int rc = build_form(s, C, pairs, t, true, true, &fits)) return rc;
+        if (fits && !long_tail) {
+            if (int rc = build_form(s, C, pairs, t, true, false, &fits)) return rc;
+            if (!own) t->panel_ok = t->pw_ok = false;
+            return DQ_OK;
+        }
+    }
+    return build_form(s, C, pairs, t, false, false, &fits);
 }
 
 }  // namespace dq
