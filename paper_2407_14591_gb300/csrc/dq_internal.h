@@ -121,6 +121,14 @@ struct PanelDiag {
     uint32_t w0[kPanelMaxK][3], w1[kPanelMaxK][3];
 };
 
+// The same for the panel kernel: the panel's constant and, per P_1 bit b, the change of the diagonal
+// when the bit is set, both / 2^emin: sum_ab K [s_a != s_b] over the cut is (sum over s_a = 1 of K) +
+// sum_b s_b w_b with w_b = sum_a K (1 - 2 s_a).
+struct PanelRowDiag {
+    long long pd;
+    long long w[15];
+};
+
 struct PanelPlan {
     int L0, L1, N;
     uint32_t npanels;
@@ -159,7 +167,8 @@ struct PanelPlan {
     const uint32_t* list_off;
     const uint32_t* list_hdr;   // bits 0-7: class-0 P_0 partners, 8-15: class-1, 16-23: crossing
     const uint64_t* list;
-    const PanelDiag* diag;      // per panel, built on the host (two subsystems)
+    const PanelRowDiag* diag;   // per panel
+    const long long* d1;        // P_1 Sz Sz of every P_1 pattern, in the order of t1states
     // three or more subsystems (the warp-panel kernel): prefix bits of the Sz Sz bonds across the
     // cut, per class and per position b of P_1 (the per-panel counters are built on the device)
     uint32_t xzA[kPanelMaxK][32];

@@ -436,30 +436,28 @@ static int build_form(const dq_sector* s, double C,
     auto start_of = [&](uint32_t p) -> uint64_t { return tail_start.empty() ? s->h.c0_tab[p] : tail_start[p]; };
     P.npanels = (uint32_t)ps0.size();
     P.cmax = cmax;
-    // per-panel diagonal counters (see PanelDiag)
-    std::vector<PanelDiag> pdiag(ps0.size());
+    // per-panel diagonal (see PanelRowDiag) and the P_1 Sz Sz sums of the patterns
+    std::vector<PanelRowDiag> pdiag(ps0.size());
     for (size_t q = 0; q < ps0.size(); ++q) {
         const uint32_t s0 = ps0[q];
-        PanelDiag& g = pdiag[q];
+        PanelRowDiag& g = pdiag[q];
         std::memset(&g, 0, sizeof g);
+        g.pd = P.MC;
         for (int k = 0; k < P.nK; ++k) {
             for (int l = (k ? P.p0z_end[k - 1] : 0); l < P.p0z_end[k]; ++l)
-                g.cnt0[k] += __builtin_popcount(s0 & P.p0z_mask[l]) == 1;
-            int c0[32] = {0}, c1[32] = {0};  // per position b of P_1: bonds with s_a = 0 / s_a = 1
+                if (__builtin_popcount(s0 & P.p0z_mask[l]) == 1) g.pd += P.MK[k];
             for (int l = (k ? P.xz_end[k - 1] : 0); l < P.xz_end[k]; ++l) {
-                const int b = __builtin_ctz(P.xz_bbit[l]);
-                if (s0 & P.xz_abit[l])
-                    ++c1[b];
-                else
-                    ++c0[b];
+                const bool sa = (s0 & P.xz_abit[l]) != 0;
+                if (sa) g.pd += P.MK[k];
+                g.w[__builtin_ctz(P.xz_bbit[l])] += sa ? -P.MK[k] : P.MK[k];
             }
-            for (int b = 0; b < 32; ++b)
-                for (int qq = 0; qq < 3; ++qq) {
-                    g.w0[k][qq] |= (uint32_t)((c0[b] >> qq) & 1) << b;
-                    g.w1[k][qq] |= (uint32_t)((c1[b] >> qq) & 1) << b;
-                }
         }
     }
+    std::vector<long long> d1(t1states.size(), 0);
+    for (size_t q = 0; q < t1states.size(); ++q)
+        for (int k = 0; k < P.nK; ++k)
+            for (int l = (k ? P.p1z_end[k - 1] : 0); l < P.p1z_end[k]; ++l)
+                d1[q] += P.MK[k] * __builtin_popcount((t1states[q] ^ (t1states[q] >> P.p1z_d[l])) & P.p1z_mask[l]);
     // per-panel source lists
     std::vector<uint32_t> loff(ps0.size() + 1, 0), lhdr(ps0.size(), 0);
     std::vector<uint64_t> lst;
@@ -502,8 +500,10 @@ static int build_form(const dq_sector* s, double C,
     P.list_hdr = (const uint32_t*)p;
     if ((rc = dev_upload(t->dev_allocs, lst.data(), lst.size() * 8, &p))) return rc;
     P.list = (const uint64_t*)p;
-    if ((rc = dev_upload(t->dev_allocs, pdiag.data(), pdiag.size() * sizeof(PanelDiag), &p))) return rc;
-    P.diag = (const PanelDiag*)p;
+    if ((rc = dev_upload(t->dev_allocs, pdiag.data(), pdiag.size() * sizeof(PanelRowDiag), &p))) return rc;
+    P.diag = (const PanelRowDiag*)p;
+    if ((rc = dev_upload(t->dev_allocs, d1.data(), d1.size() * 8, &p))) return rc;
+    P.d1 = (const long long*)p;
     P.c0 = s->dev.c0_tab;
     if (split) {
         // canonical order of the rows of a panel (see the file comment)

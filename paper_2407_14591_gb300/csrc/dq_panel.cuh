@@ -98,19 +98,21 @@ __device__ __forceinline__ int stage(XT* buf, const XT* X, uint64_t start, int l
 //   kOwn + s * bstride, s < R: R slots of cap + 8 elements. Slot 0 holds the panel's own x, slots
 //                  1 .. R-1 are the ring of cut partners. Elements cap - 1 .. cap + 6 of every
 //                  slot stay zero (no copy reaches them).
-//   then R mbarriers and the panel's source list.
+//   then R mbarriers, the source lists of the panel and of the next one, and the panel's diagonal sums:
+//   256 by the low eight P_1 bits (the panel's constant in each), 128 by the others.
 // A table entry is a byte offset into a slot, so a gather is two loads with no address arithmetic.
 constexpr int kT1Entries = 1 << 15;
 constexpr uint32_t kZeroSlot = 2 * kT1Entries;  // byte offset of the zero-slot entry
 constexpr int kT1Bytes = 2 * kT1Entries + 128;
 constexpr int kOwn = kT1Bytes;
 constexpr int kZeroPad = 8;
+constexpr int kDiagLow = 256, kDiagSums = kDiagLow + 128;
 template <typename XT>
 struct PanelSmem {
     static __host__ __device__ size_t al(size_t b) { return (b + 127) & ~(size_t)127; }
     static __host__ __device__ size_t buf_bytes(int cap) { return al((size_t)(cap + kZeroPad) * sizeof(XT)); }
     static __host__ __device__ size_t total(int cap, int nslots) {
-        return kT1Bytes + (size_t)nslots * buf_bytes(cap) + 128 + 8 * kPanelMaxList;
+        return kT1Bytes + (size_t)nslots * buf_bytes(cap) + 128 + 2 * 8 * kPanelMaxList + 8 * kDiagSums;
     }
 };
 
@@ -126,6 +128,12 @@ struct PanelCtx {
     uint32_t s0;
     uint64_t start, piece;
     int n1, C, ncls0, np0, nx;
+};
+
+// What a block reads of a panel one panel ahead.
+struct PanelHead {
+    uint64_t start;
+    uint32_t s0, hdr;
 };
 
 // Block-shared bookkeeping of the copy ring.
@@ -170,7 +178,7 @@ __device__ __forceinline__ void release_slot(int s, int jn, const PanelPlan& P, 
 // gathers read in-range entries, and they are never stored.
 template <typename XT, typename OUT, int NA, int R, int E, int NT, bool SPLIT>
 __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restrict__ X, OUT* __restrict__ y,
-                                           unsigned char* smem, uint64_t* bar, const uint64_t* lst, const PanelDiag& dg,
+                                           unsigned char* smem, uint64_t* bar, const uint64_t* lst, const long long* sums,
                                            const PanelCtx& pc, size_t bstride, uint32_t& ph, int scale, int& fail,
                                            Ring<R>& rg) {
     const int tid = threadIdx.x;
@@ -300,24 +308,16 @@ __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restr
         for (; u < target; ++u) run_unit(u);
     }
     for (; u < nu; ++u) run_unit(u);
-    // the row result: (C + sum_k K_k n_k) x_i + sum_k A_k S_k, exactly, rounded once
-    const uint32_t m1 = (1u << P.L1) - 1u;
+    // the row result: (diagonal) x_i + sum_k A_k S_k, exactly, rounded once. The diagonal is the
+    // pattern's P_1 Sz Sz sum (a table) and the panel's two sums (its constant and the cut bonds)
+    // (6 x 5 lattice, N = 15: counting the bonds per row took 0.7 ms of 13.3 in FP64, 0.9 of 10.0 in FP32)
+    const long long* d1 = P.d1 + P.t1start[pc.n1];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         int c = tid + e * NT;
         if (c >= pc.C) continue;
         const uint32_t s = s2[e] >> 1;
-        long long md = P.MC;
-#pragma unroll
-        for (int k = 0; k < kPanelMaxK; ++k) {
-            if (k >= P.nK) break;
-            long long n = dg.cnt0[k];
-            for (int l = (k ? P.p1z_end[k - 1] : 0); l < P.p1z_end[k]; ++l)
-                n += __popc((s ^ (s >> P.p1z_d[l])) & P.p1z_mask[l]);
-#pragma unroll
-            for (int q = 0; q < 3; ++q) n += (long long)(__popc(s & dg.w0[k][q]) + __popc(~s & m1 & dg.w1[k][q])) << q;
-            md += P.MK[k] * n;
-        }
+        const long long md = __ldg(d1 + c) + sums[s & (kDiagLow - 1)] + sums[kDiagLow + (s >> 8)];
         I128 r = {0, 0};
         mac(r, md, lds_x<XT>(own, (uint32_t)(c * sizeof(XT))));
 #pragma unroll
@@ -344,9 +344,9 @@ __global__ void __launch_bounds__(NT, kPT / NT)
     unsigned char* tail = smem + kOwn + (size_t)R * bstride;
     uint64_t* bar = reinterpret_cast<uint64_t*>(tail);  // [s]: copy slot s
     uint64_t* lst = reinterpret_cast<uint64_t*>(tail + 128);
-    __shared__ uint32_t s_hdr;
+    long long* sums = reinterpret_cast<long long*>(tail + 128 + 2 * 8 * kPanelMaxList);
+    __shared__ PanelHead next;
     __shared__ int s_fail;
-    __shared__ PanelDiag dg;
     __shared__ Ring<R> rg;
     const uint16_t zoff = (uint16_t)((cap - 1) * sizeof(XT));  // byte offset of a zero element
 
@@ -377,60 +377,75 @@ __global__ void __launch_bounds__(NT, kPT / NT)
     uint32_t ph = 0u;  // mbarrier parity of each slot (bit s)
     int fail = 0;
 
+    // The head and the source list of a panel are read one panel ahead (by the last warp, into `next`),
+    // so that its copies start without a chain of dependent loads.
+    auto fetch = [&](uint32_t pi) {
+        if (tid < NT - 32 || pi >= P.npanels) return;
+        const int lane = tid & 31;
+        const uint32_t lo = __ldg(P.list_off + pi), hi = __ldg(P.list_off + pi + 1);
+        for (uint32_t q = lo + lane; q < hi; q += 32) lst[kPanelMaxList + q - lo] = __ldg(P.list + q);
+        if (lane == 0) {
+            next.s0 = __ldg(P.panel_s0 + pi);
+            next.start = __ldg(P.panel_start + pi);
+            next.hdr = __ldg(P.list_hdr + pi);
+        }
+    };
+    fetch(blockIdx.x);
     for (uint32_t pi = blockIdx.x; pi < P.npanels; pi += gridDim.x) {
+        __syncthreads();  // the previous panel is finished, the next one's head and list are there
         PanelCtx pc;
-        pc.s0 = P.panel_s0[pi];
-        pc.start = P.panel_start[pi];
+        pc.s0 = next.s0;
+        pc.start = next.start;
         pc.n1 = P.N - __popc(pc.s0);
         pc.C = (int)P.t1len[pc.n1];
         if constexpr (SPLIT) pc.piece = (uint64_t)pi * P.npiece;
-        // warp 0: source list into shared memory and the first copies; warp 1: diagonal counters
+        {
+            const uint32_t hd = next.hdr;
+            pc.ncls0 = (int)(hd & 255u);
+            pc.np0 = pc.ncls0 + (int)((hd >> 8) & 255u);
+            pc.nx = (int)((hd >> 16) & 255u);
+        }
         if (tid < 32) {
-            const uint32_t lo = __ldg(P.list_off + pi), hi = __ldg(P.list_off + pi + 1);
-            for (uint32_t q = lo + tid; q < hi; q += 32) lst[q - lo] = __ldg(P.list + q);
-            if (tid == 0) s_hdr = __ldg(P.list_hdr + pi);
+            for (int q = tid; q < pc.np0 + pc.nx; q += 32) lst[q] = lst[kPanelMaxList + q];
             __syncwarp();
-            if (tid == 0) {
-                const uint32_t hd = s_hdr;
-                PanelCtx pq = pc;
-                pq.np0 = (int)(hd & 255u) + (int)((hd >> 8) & 255u);
-                pq.nx = (int)((hd >> 16) & 255u);
-                for (int j = 0; j < pq.nx && j < R - 1; ++j)
-                    issue_cut<XT, R>(j, 1 + j, P, pq, X, smem, bstride, bar, lst, rg);
-            }
-        } else if (tid < 32 + (int)(sizeof(PanelDiag) / 4)) {
-            // the panel's diagonal counters, built on the host
-            reinterpret_cast<uint32_t*>(&dg)[tid - 32] = __ldg(reinterpret_cast<const uint32_t*>(P.diag + pi) + tid - 32);
+            if (tid == 0)
+                for (int j = 0; j < pc.nx && j < R - 1; ++j)
+                    issue_cut<XT, R>(j, 1 + j, P, pc, X, smem, bstride, bar, lst, rg);
         }
         // the panel's own x: plain coalesced loads into slot 0 (element c at kOwn + c*size)
         {
             const XT* src = X + pc.start;
             for (int c = tid; c < pc.C; c += NT) own[c] = __ldg(src + c);
         }
+        if (tid < kDiagSums) {
+            const long long* w = P.diag[pi].w + (tid < kDiagLow ? 0 : 8);
+            const int bits = tid < kDiagLow ? 8 : 7;
+            long long sum = tid < kDiagLow ? __ldg(&P.diag[pi].pd) : 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q < bits && ((tid >> q) & 1)) sum += __ldg(w + q);
+            sums[tid] = sum;
+        }
         __syncthreads();
-        const uint32_t hd = s_hdr;
-        pc.ncls0 = (int)(hd & 255u);
-        pc.np0 = pc.ncls0 + (int)((hd >> 8) & 255u);
-        pc.nx = (int)((hd >> 16) & 255u);
+        fetch(pi + gridDim.x);
         // rows per thread: the smallest E with E * NT >= C (every E from 1 to 7 is compiled for
         // 1024 threads; 512-thread CTAs take panels of at most 1024 rows)
         if constexpr (NT == kPT) {
             switch ((pc.C + NT - 1) / NT) {
-                case 7: panel_rows<XT, OUT, NA, R, 7, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg); break;
-                case 6: panel_rows<XT, OUT, NA, R, 6, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg); break;
-                case 5: panel_rows<XT, OUT, NA, R, 5, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg); break;
-                case 4: panel_rows<XT, OUT, NA, R, 4, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg); break;
-                case 3: panel_rows<XT, OUT, NA, R, 3, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg); break;
-                case 2: panel_rows<XT, OUT, NA, R, 2, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg); break;
-                default: panel_rows<XT, OUT, NA, R, 1, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg);
+                case 7: panel_rows<XT, OUT, NA, R, 7, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 6: panel_rows<XT, OUT, NA, R, 6, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 5: panel_rows<XT, OUT, NA, R, 5, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 4: panel_rows<XT, OUT, NA, R, 4, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 3: panel_rows<XT, OUT, NA, R, 3, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 2: panel_rows<XT, OUT, NA, R, 2, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                default: panel_rows<XT, OUT, NA, R, 1, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
             }
         } else {
             if (pc.C > NT)
-                panel_rows<XT, OUT, NA, R, 2, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg);
+                panel_rows<XT, OUT, NA, R, 2, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
             else
-                panel_rows<XT, OUT, NA, R, 1, NT, SPLIT>(P, X, y, smem, bar, lst, dg, pc, bstride, ph, scale, fail, rg);
+                panel_rows<XT, OUT, NA, R, 1, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
         }
-        __syncthreads();
     }
     if (fail) s_fail = 1;
     __syncthreads();
