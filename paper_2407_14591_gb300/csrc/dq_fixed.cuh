@@ -130,6 +130,46 @@ __device__ __forceinline__ OUT i128_to(I128 a, int scale) {
     }
 }
 
+// ------------------------------------------------------------------ split products ----------
+
+// A 57-bit X stored as one 64-bit word whose high half is X_h = X >> 28 (signed) and whose low half is
+// X_l = X mod 2^28, so that X = X_h 2^28 + X_l. With a coefficient split the same way, a product is four
+// 32 x 32 -> 64-bit multiply-adds into three int64 sums instead of a 64 x 64 -> 128-bit one.
+__device__ __forceinline__ long long split_word(long long v) {
+    return (long long)(((unsigned long long)(uint32_t)(int)(v >> 28) << 32) | (unsigned long long)(v & 0xfffffffll));
+}
+__device__ __forceinline__ long long join_word(long long w) {
+    return (long long)(int)(w >> 32) * (1ll << 28) + (long long)(w & 0xffffffffll);
+}
+
+struct Acc3 {
+    long long hh, mid, ll;
+};
+
+// d = a b + c with the signed 32 x 32 -> 64-bit product (one mad.wide.s32; the same sum written
+// with 64-bit operands in C++ took about a fifth longer on workload 3)
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ void acc_hop(Acc3& a, int2 m, long long xs) {
+    const int xh = (int)(xs >> 32), xl = (int)(xs & 0xffffffffll);
+    a.hh = mad_wide(m.x, xh, a.hh);
+    a.mid = mad_wide(m.y, xh, mad_wide(m.x, xl, a.mid));
+    a.ll = mad_wide(m.y, xl, a.ll);
+}
+
+// a += v 2^sh for 0 <= sh < 64
+__device__ __forceinline__ void add_shifted(I128& a, long long v, int sh) {
+    const unsigned long long lo = sh ? (unsigned long long)v << sh : (unsigned long long)v;
+    const long long hi = sh ? (v >> (64 - sh)) : (v >> 63);
+    const unsigned long long s = a.lo + lo;
+    a.hi += hi + (s < a.lo ? 1 : 0);
+    a.lo = s;
+}
+
 // ------------------------------------------------------------------ per-column prepass -------
 
 // Scales of an interleaved block of nrhs <= 64 columns (x[i * nrhs + c]).

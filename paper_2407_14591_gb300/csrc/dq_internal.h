@@ -227,24 +227,24 @@ struct PanelPB {
     const uint16_t* t1rank;       // local index of every P_1 pattern
     const uint16_t* t1states;     // P_1 patterns grouped by particle number
     uint32_t t1start[kPBMaxL1 + 2], t1len[kPBMaxL1 + 2];
-    // bonds inside P_1: pair mask (bits lo, hi), hop amplitude and Sz Sz coefficient (device)
+    // hop bonds inside P_1: bit of the lower position, distance, pair mask, all shifted left by one
+    // (byte offsets into the rank table)
     int n1b;
-    uint32_t p1_lo[kPBMaxBonds], p1_hi[kPBMaxBonds];
-    const long long* p1_A;        // [n1b]
-    const long long* p1_K;        // [n1b]
-    // bonds across the cut, grouped by the P_0 bit a (partner panel s0 ^ a): P_1 bit b and
-    // coefficients; groups with a hop amplitude only (the Sz Sz parts are in xz_*)
-    int nxg;
+    uint32_t p1_lo2[kPBMaxBonds], p1_pm2[kPBMaxBonds];
+    int p1_d[kPBMaxBonds];
+    // hop bonds across the cut, grouped by the P_0 bit a (partner panel s0 ^ a): P_1 bit b, shifted
+    // left by one
+    int nxg, nvis;
     uint32_t xg_abit[kPBMaxGroups];
     int xg_first[kPBMaxGroups], xg_end[kPBMaxGroups];
-    uint32_t xb_bit[kPBMaxBonds];
-    const long long* xb_A;        // [bonds]
-    int nxz;                       // Sz Sz bonds across the cut: [s_a != s_b] with coefficient K
-    uint32_t xz_abit[kPBMaxBonds], xz_bbit[kPBMaxBonds];
-    const long long* xz_K;
-    const long long* f1;          // [L1]: field of P_1 bit b (coefficient of s_b)
-    const long long* pdiag;       // per panel: constant + P_0 fields + P_0 Sz Sz bonds
-    const long long* p0_A;        // hop amplitude of each P_0 bond (index in the partner entry)
+    uint32_t xb_bit2[kPBMaxBonds];
+    // hop amplitudes, split as M = x 2^28 + y with |y| <= 2^27: the P_1 bonds, the cut bonds, the P_0
+    // bonds (index in the partner entry)
+    const int2* amp;
+    int namp;
+    const long long* d1;          // P_1 fields and Sz Sz of every P_1 pattern, in the order of t1states
+    const PanelRowDiag* pdiag;    // per panel
+    bool flush;                   // more hops per row than the split sums hold
     // per-panel sources: P_0 partners (start | bond << 48) then cross partners (start | group << 48)
     const uint32_t* list_off;
     const uint32_t* list_hdr;     // bits 0-7: P_0 partners, 8-15: cross partners
@@ -356,7 +356,7 @@ int launch_index_of_batch_w(const DevSector& S, const uint64_t* d_state, uint64_
 // (K of [s_lo != s_hi], hop amplitude A), per-position fields and the constant
 int build_panel_pb(const dq_sector* s, double C, const double* lin,
                    const std::vector<std::pair<std::pair<int, int>, std::pair<double, double>>>& pairs, dq_terms* t);
-int launch_panel_pb(const dq_sector* s, dq_terms* t, const void* x, void* y, int dtype, void* stream);
+int launch_panel_pb(const dq_sector* s, dq_terms* t, const void* x, void* y, int dtype, int cols, void* stream);
 
 // validation shared by the term compilers (dq_terms.cpp): DQ_OK or the error status
 int check_terms(const dq_sector* s, const dq_term* terms, int n_terms);

@@ -249,34 +249,6 @@ __global__ void k_split_fixed(const T* __restrict__ x, long long* __restrict__ X
     }
 }
 
-struct Acc3 {
-    long long hh, mid, ll;
-};
-
-// d = a b + c with the signed 32 x 32 -> 64-bit product (one mad.wide.s32; the same sum written
-// with 64-bit operands in C++ took about a fifth longer on workload 3)
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
-    long long d;
-    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ void acc_hop(Acc3& a, int2 m, long long xs) {
-    const int xh = (int)(xs >> 32), xl = (int)(xs & 0xffffffffll);
-    a.hh = mad_wide(m.x, xh, a.hh);
-    a.mid = mad_wide(m.y, xh, mad_wide(m.x, xl, a.mid));
-    a.ll = mad_wide(m.y, xl, a.ll);
-}
-
-// a += v 2^sh for 0 <= sh < 64
-__device__ __forceinline__ void add_shifted(I128& a, long long v, int sh) {
-    const unsigned long long lo = sh ? (unsigned long long)v << sh : (unsigned long long)v;
-    const long long hi = sh ? (v >> (64 - sh)) : (v >> 63);
-    const unsigned long long s = a.lo + lo;
-    a.hi += hi + (s < a.lo ? 1 : 0);
-    a.lo = s;
-}
-
 constexpr int kPQT = 512;           // threads per CTA
 constexpr int kPQW = kPQT / 32;     // warps per CTA, one panel each at a time
 

@@ -108,3 +108,36 @@ def test_workload5_full_size():
     assert t.path == "panel_pb"
     o = OracleSector(w.L, w.Q, w.N, partition=s.partition)
     check(s, t, w.terms, o, x)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("cols", [2, 3])
+def test_columns_equal_single_products(cols, dtype):
+    """Two and three right-hand sides (one launch over panels and columns, D = 705,432) equal the same
+    columns one by one: same integers per column, whatever the other columns' scales are."""
+    rng = np.random.default_rng(cols)
+    L = 22
+    s = b.make_sector(L, 2, 11, 2)
+    t = b.make_terms(s, disordered_terms(rng, wl.chain_bonds(L), L))
+    x = torch.from_numpy(rng.uniform(-1, 1, (s.dim, cols)) * 10.0 ** np.arange(-3, cols - 3)).to(DEV, dtype)
+    y = b.matvec(s, t, x, torch.full_like(x, float("nan")))
+    for c in range(cols):
+        assert torch.equal(y[:, c], b.matvec(s, t, x[:, c].contiguous()))
+    x[5, cols - 1] = float("inf")
+    assert torch.isnan(b.matvec(s, t, x)).all()
+    with pytest.raises(b.DQError):
+        s.check_device()
+
+
+def test_many_hops_per_row():
+    """A ring of 16 sites coupled up to distance six, whose rows can hop more than 63 times: the sums
+    are carried into 128 bits on the way."""
+    rng = np.random.default_rng(7)
+    L = 16
+    bonds = [(i, (i + d) % L) for i in range(L) for d in (1, 2, 3, 4, 5, 6)]
+    terms = disordered_terms(rng, bonds, L)
+    s = b.make_sector(L, 2, 8, 2)
+    t = b.make_terms(s, terms)
+    assert t.path == "panel_pb"
+    o = OracleSector(L, 2, 8, partition=s.partition)
+    check(s, t, terms, o, rng.uniform(-1, 1, o.dim))
