@@ -24,6 +24,7 @@
 
 #include "dq_device.cuh"
 #include "dq_fixed.cuh"
+#include "dq_grad.h"
 #include "dq_internal.h"
 
 namespace dq {
@@ -226,6 +227,20 @@ __global__ void k_grad_finish(const double* __restrict__ partial, int nb, double
     out[u] = v;
 }
 
+int grad_workspace(const dq_sector* s, size_t need, char** ws) {
+    dq_sector* sw = const_cast<dq_sector*>(s);
+    if (sw->grad_ws_bytes < need) {
+        if (sw->grad_ws) cudaFree(sw->grad_ws);
+        sw->grad_ws = nullptr;
+        sw->grad_ws_bytes = 0;
+        const cudaError_t e = cudaMalloc(&sw->grad_ws, need);
+        if (e != cudaSuccess) return (int)e;
+        sw->grad_ws_bytes = need;
+    }
+    *ws = reinterpret_cast<char*>(sw->grad_ws);
+    return 0;
+}
+
 }  // namespace dq
 
 using namespace dq;
@@ -253,6 +268,18 @@ extern "C" int dq_term_grads(const dq_sector* s, const dq_term* terms, int n_ter
         gt[q].sh_i = s->nb * (s->L - 1 - u.i);
         gt[q].sh_j = pair ? s->nb * (s->L - 1 - u.j) : -1;
     }
+    cudaStream_t st = (cudaStream_t)stream;
+    {
+        bool taken = false;
+        cudaError_t pe = (cudaError_t)launch_grad_panel(s, terms, n_terms, x, dy, dtype, nrhs, d_grads, st, &taken);
+        if (taken) {
+            if (pe == cudaErrorMemoryAllocation)
+                return set_error(DQ_ENOMEM, "term gradients workspace: %s", cudaGetErrorString(pe));
+            if (pe == cudaSuccess) pe = cudaStreamSynchronize(st);
+            if (pe != cudaSuccess) return set_error(DQ_ECUDA, "term gradients: %s", cudaGetErrorString(pe));
+            return DQ_OK;
+        }
+    }
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -273,18 +300,9 @@ extern "C" int dq_term_grads(const dq_sector* s, const dq_term* terms, int n_ter
     const size_t o_x = o_part + al(sizeof(double) * kGradChunk * nb);
     const size_t vec = fx ? al((size_t)s->D * nrhs * sizeof(long long)) : 0;
     const size_t need = o_x + 2 * vec;
-    dq_sector* sw = const_cast<dq_sector*>(s);
-    cudaError_t e = cudaSuccess;
-    if (sw->grad_ws_bytes < need) {
-        if (sw->grad_ws) cudaFree(sw->grad_ws);
-        sw->grad_ws = nullptr;
-        sw->grad_ws_bytes = 0;
-        e = cudaMalloc(&sw->grad_ws, need);
-        if (e != cudaSuccess) return set_error(DQ_ENOMEM, "term gradients workspace (%zu bytes): %s", need,
-                                               cudaGetErrorString(e));
-        sw->grad_ws_bytes = need;
-    }
-    char* ws = reinterpret_cast<char*>(sw->grad_ws);
+    char* ws = nullptr;
+    cudaError_t e = (cudaError_t)grad_workspace(s, need, &ws);
+    if (e != cudaSuccess) return set_error(DQ_ENOMEM, "term gradients workspace (%zu bytes): %s", need, cudaGetErrorString(e));
     ColScale* hx = reinterpret_cast<ColScale*>(ws);
     ColScale* hdy = reinterpret_cast<ColScale*>(ws + o_hdy);
     GradTerm* d_gt = reinterpret_cast<GradTerm*>(ws + o_gt);
@@ -292,7 +310,6 @@ extern "C" int dq_term_grads(const dq_sector* s, const dq_term* terms, int n_ter
     double* d_part = reinterpret_cast<double*>(ws + o_part);
     long long* X = reinterpret_cast<long long*>(ws + o_x);
     long long* DYf = reinterpret_cast<long long*>(ws + o_x + vec);
-    cudaStream_t st = (cudaStream_t)stream;
     e = cudaMemcpyAsync(d_gt, gt.data(), sizeof(GradTerm) * n_terms, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_amp, amp.data(), sizeof(double) * amp.size(), cudaMemcpyHostToDevice, st);
     const bool use_sm = (size_t)s->dev.os_total * 16 <= 48 * 1024;
