@@ -80,6 +80,13 @@ __device__ __forceinline__ uint64_t d_rank_within(const DevSector& S, const uint
     return checked_rank(S, i + (uint64_t)((long long)st * delta));
 }
 
+// idx / st for st > 0; with both below 2^32, as in all but the largest sectors, by the 32-bit division
+// (a 64-bit one is several times as long).
+__device__ __forceinline__ uint64_t d_quot(uint64_t idx, uint64_t st) {
+    if (((idx | st) >> 32) == 0) return (uint32_t)idx / (uint32_t)st;
+    return idx / st;
+}
+
 // Alg. 4 for idx < D.
 template <typename W = uint64_t>
 __device__ __forceinline__ W d_unrank(const DevSector& S, const uint64_t* off_s, const uint64_t* str_s, uint64_t idx) {
@@ -98,7 +105,7 @@ __device__ __forceinline__ W d_unrank(const DevSector& S, const uint64_t* off_s,
             while (n < S.nmax[k] && !(idx < off_s[base + n + 1])) ++n;
             idx -= off_s[base + n];
             uint64_t st = str_s[base + n];
-            li = idx / st;
+            li = d_quot(idx, st);
             idx -= li * st;
         }
         int t = S.tab[k];
@@ -134,7 +141,7 @@ __device__ __forceinline__ void walk_start(const DevSector& S, const uint64_t* o
         while (n < S.nmax[k] && !(idx < off_s[base + n + 1])) ++n;
         idx -= off_s[base + n];
         const uint64_t st = str_s[base + n];
-        const uint64_t li = idx / st;
+        const uint64_t li = d_quot(idx, st);
         idx -= li * st;
         const int t = S.tab[k];
         w |= (W)__ldg(S.unrank_tab[t] + __ldg(S.sec_start[t] + n) + li) << S.shift[k];
@@ -168,14 +175,13 @@ __device__ __forceinline__ bool d_valid(const DevSector& S, W w) {
     constexpr int WB = 8 * (int)sizeof(W);
     int bits = S.L * S.nb;
     if (bits < WB && (w >> bits) != 0) return false;
+    if (S.nb == 1) return popc_w(w) == S.N;
     if ((S.Q & (S.Q - 1)) == 0) {
         // Q = 2^Nbits: every digit is < Q; the digit sum is a weighted popcount of bit planes
+        W plane = S.nb == 2 ? (W)0x5555555555555555ull : S.nb == 3 ? (W)0x9249249249249249ull : (W)0x1111111111111111ull;
+        if (WB > 64) plane |= (S.nb == 3 ? (W)0x4924924924924924ull : plane) << (WB > 64 ? 64 : 0);
         int n = 0;
-        for (int b = 0; b < S.nb; ++b) {
-            W plane = 0;
-            for (int q = b; q < WB; q += S.nb) plane |= (W)1 << q;
-            n += popc_w(w & plane) << b;
-        }
+        for (int b = 0; b < S.nb; ++b) n += popc_w(w & (plane << b)) << b;
         return n == S.N;
     }
     int n = 0;

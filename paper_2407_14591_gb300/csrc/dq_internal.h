@@ -345,6 +345,9 @@ uint64_t host_rank(const dq_sector* s, u128 w);
 u128 host_unrank(const dq_sector* s, uint64_t idx);
 
 // kernel launchers (dq_kernels.cu); return a cudaError_t as int
+// Rank (inverse: unrank) of a long list with the tables in shared memory (dq_rank.cu). 0: launched; -1: not
+// a list or sector for it, nothing launched; otherwise a CUDA error.
+int launch_rank_long(const DevSector& S, bool inverse, const uint64_t* in, uint64_t* out, uint64_t n, cudaStream_t st);
 int launch_state_at_batch(const DevSector& S, const uint64_t* d_index, uint64_t* d_state, uint64_t n, void* stream);
 int launch_index_of_batch(const DevSector& S, const uint64_t* d_state, uint64_t* d_index, uint64_t n, void* stream);
 int launch_matvec(const dq_sector* s, const dq_terms* t, const void* x, void* y, int dtype, int nrhs, void* stream);

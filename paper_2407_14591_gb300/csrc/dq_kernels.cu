@@ -316,12 +316,14 @@ static void launch_resident(void (*kernel)(KArgs...), uint64_t rows, size_t smb,
 }
 
 int launch_state_at_batch(const DevSector& S, const uint64_t* d_index, uint64_t* d_state, uint64_t n, void* stream) {
+    if (const int e = launch_rank_long(S, true, d_index, d_state, n, (cudaStream_t)stream); e >= 0) return e;
     bool sm = os_in_smem(S);
     k_state_at<<<grid_for(n, 256, 8), 256, sm ? os_bytes(S) : 0, (cudaStream_t)stream>>>(S, d_index, d_state, n, sm);
     return (int)cudaGetLastError();
 }
 
 int launch_index_of_batch(const DevSector& S, const uint64_t* d_state, uint64_t* d_index, uint64_t n, void* stream) {
+    if (const int e = launch_rank_long(S, false, d_state, d_index, n, (cudaStream_t)stream); e >= 0) return e;
     bool sm = os_in_smem(S);
     k_index_of<<<grid_for(n, 256, 8), 256, sm ? os_bytes(S) : 0, (cudaStream_t)stream>>>(S, d_state, d_index, n, sm);
     return (int)cudaGetLastError();
