@@ -270,14 +270,18 @@ struct PanelQ {
     const long long* Mhop;        // [bonds][Q][Q]: -t sqrt((n_up + 1) n_dn) on the grid 2^emin; entry nM is 0
     // per P_1 pattern (index t1start[n1] + local index c):
     const long long* rdiag;       // the P_1 site functions
-    const uint32_t* p1ell;        // from p1base[n1], p1m[n1] slots of C entries: partner | Mhop entry << 16
-    uint32_t p1base[kPQMaxN + 1], p1m[kPQMaxN + 1];
+    const uint32_t* p1ell;        // from p1base[n1], slots of C entries: partner | Mhop entry << 16
+    const unsigned char* p1cnt;   // from p1cbase[n1], per 32 patterns: slots in use
+    uint32_t p1base[kPQMaxN + 1], p1cbase[kPQMaxN + 1];
     const uint32_t* cutt;         // from cutbase[n1], ncut slots of C entries: partner local index |
                                   // row part of the Mhop entry << 16 | (the hop is not allowed) << 31
     uint32_t cutbase[kPQMaxN + 1];
     const long long* pdiag;       // per panel: the constant plus the P_0 site functions
     // per-panel sources: P_0 partners (start | Mhop entry << 40), then cut partners
     // (start | cut direction << 40 | panel part of the Mhop entry << 48)
+    // work of a warp: panel | first 32-row chunk << 32 | chunks << 48 | the next panel too << 63
+    const uint64_t* unit;
+    uint32_t nunits, pairs;       // pairs: units are of two panels
     const uint32_t* list_off;
     const uint32_t* list_hdr;     // bits 0-7: P_0 entries, 8-15: cut entries
     const uint64_t* list;

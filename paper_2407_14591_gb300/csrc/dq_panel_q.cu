@@ -20,8 +20,14 @@
 // four 32 x 32 -> 64-bit products (below). Every row is one exact integer sum rounded once; the
 // coefficients are those of the general kernel, so on FP64 vectors the two give the same y.
 //
-// One warp per panel: the warps of persistent 512-thread CTAs take panels from an atomic counter,
-// longest panels first, and never wait for each other; a warp's lanes take the panel's rows.
+// The warps of persistent 512-thread CTAs take units from an atomic counter, longest first, and never
+// wait for each other; a warp's lanes take the rows. A unit is a piece of a few 32-row chunks of one panel or
+// of TWO panels with the same particle number: the tables of P_1 depend on the row's P_1 pattern only, so
+// both panels share each table entry and amplitude that is read. Pieces even out the warps' work: a whole
+// panel of the largest block (2128 rows on the 14-site chain with four levels and 14 bosons) is more than a
+// warp's share of the sector (1330 rows). That chain, FP32: 277 -> 229 us per product (whole panels singly
+// before), FP64 290 -> 246. A chunk's rows use as many P_1 slots as the longest of their lists: 9.0 a row
+// instead of the block's 11.1, 6.3 of them real. Bound: instruction issue.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -35,6 +41,9 @@
 namespace dq {
 
 constexpr uint64_t kPQStart = (1ull << 40) - 1;
+constexpr uint32_t kPQChunks = 4;  // 32-row chunks of a unit, at most
+constexpr int kPQT = 512;          // threads per CTA
+constexpr int kPQW = kPQT / 32;    // warps per CTA, one unit each at a time
 
 // ------------------------------------------------------------------ plan (host) -------------
 
@@ -92,6 +101,7 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
     const size_t npat = ut.size();
     std::vector<long long> rdiag(npat, 0);
     std::vector<uint32_t> p1ell, cutt;
+    std::vector<unsigned char> p1cnt;
     for (int n = 0; n <= n1max; ++n) {
         const uint32_t C1 = P.t1len[n], b0 = P.t1start[n];
         std::vector<std::vector<uint32_t>> lists(C1);
@@ -111,7 +121,12 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
             mx = std::max(mx, lists[c].size());
         }
         P.p1base[n] = (uint32_t)p1ell.size();
-        P.p1m[n] = (uint32_t)mx;
+        P.p1cbase[n] = (uint32_t)p1cnt.size();
+        for (uint32_t c = 0; c < C1; c += 32) {  // slots that the rows of a chunk use (lists are left-aligned)
+            size_t m = 0;
+            for (uint32_t q = c; q < C1 && q < c + 32; ++q) m = std::max(m, lists[q].size());
+            p1cnt.push_back((unsigned char)m);
+        }
         for (size_t m = 0; m < mx; ++m)  // padding: the row itself with the zero amplitude nM
             for (uint32_t c = 0; c < C1; ++c)
                 p1ell.push_back(m < lists[c].size() ? lists[c][m] : (c | ((uint32_t)P.nM << 16)));
@@ -195,6 +210,39 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
         lhdr[i] = n0e | (nxe << 8);
     }
     loff[pl.size()] = (uint32_t)lst.size();
+    // Units: panels in pairs of neighbours with the same particle number (an odd one out with itself) or
+    // single, cut into pieces, full pieces first. The pieces are as long as leaves every resident warp four
+    // units, and the panels are paired while it leaves one: on smaller sectors a unit's length is the
+    // product's time (44,473 rows: pieces of 4, 2 chunks of pairs 36, 28 us; 8451 rows: pairs 24, single 20 us).
+    auto n_of = [&](uint32_t s0) {
+        int n = 0;
+        for (int k = 0; k < L0; ++k) n += digit0(s0, nb * k);
+        return n;
+    };
+    std::vector<uint64_t> units;
+    auto cut = [&](bool pair, uint32_t chunks) {
+        std::vector<std::vector<uint64_t>> unit(chunks + 1);
+        for (size_t i = 0; i < pl.size();) {
+            const bool two = pair && i + 1 < pl.size() && n_of(ps0[i]) == n_of(ps0[i + 1]);
+            const uint32_t ch = (~pl[i].first.first + 31) / 32;
+            for (uint32_t c = 0; c < ch; c += chunks) {
+                const uint32_t len = std::min(chunks, ch - c);
+                unit[len].push_back((uint64_t)i | ((uint64_t)c << 32) | ((uint64_t)len << 48) | ((uint64_t)two << 63));
+            }
+            i += two ? 2 : 1;
+        }
+        units.clear();
+        for (uint32_t len = chunks; len > 0; --len) units.insert(units.end(), unit[len].begin(), unit[len].end());
+    };
+    const size_t warps = (size_t)sm_count_cached() * 2 * kPQW;
+    uint32_t chunks = kPQChunks;
+    P.pairs = 1;
+    for (cut(true, chunks); chunks > 1 && units.size() < 4 * warps; cut(true, chunks)) chunks /= 2;
+    if (units.size() < warps) {
+        P.pairs = 0;
+        cut(false, chunks);
+    }
+    P.nunits = (uint32_t)units.size();
     int rc;
     void* p;
     auto up = [&](const void* src, size_t bytes, const void** dst) -> int {
@@ -214,6 +262,8 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
     if ((rc = up(rdiag.data(), rdiag.size() * 8, (const void**)&P.rdiag))) return rc;
     if ((rc = up(p1ell.data(), p1ell.size() * 4, (const void**)&P.p1ell))) return rc;
     if ((rc = up(cutt.data(), cutt.size() * 4, (const void**)&P.cutt))) return rc;
+    if ((rc = up(units.data(), units.size() * 8, (const void**)&P.unit))) return rc;
+    if ((rc = up(p1cnt.data(), p1cnt.size(), (const void**)&P.p1cnt))) return rc;
     if ((rc = up(pdiag.data(), pdiag.size() * 8, (const void**)&P.pdiag))) return rc;
     if ((rc = up(loff.data(), loff.size() * 4, (const void**)&P.list_off))) return rc;
     if ((rc = up(lhdr.data(), lhdr.size() * 4, (const void**)&P.list_hdr))) return rc;
@@ -249,21 +299,19 @@ __global__ void k_split_fixed(const T* __restrict__ x, long long* __restrict__ X
     }
 }
 
-constexpr int kPQT = 512;           // threads per CTA
-constexpr int kPQW = kPQT / 32;     // warps per CTA, one panel each at a time
-
-// Shared memory: the split amplitudes (int2 per Mhop entry, the zero entry nM last) and one
-// source-list slot per warp.
+// Shared memory: the split amplitudes (int2 per Mhop entry, the zero entry nM last) and the source lists of
+// one unit per warp.
 struct PQSmem {
     size_t ms, lst, total;
     __host__ __device__ PQSmem(const PanelQ& P) {
         ms = 0;
         lst = ((size_t)(P.nM + 1) * 8 + 15) & ~(size_t)15;
-        total = lst + (size_t)8 * kPQMaxList * kPQW;
+        total = lst + (size_t)16 * kPQMaxList * kPQW;
     }
 };
 
-template <typename OUT>
+// NP: panels of a unit.
+template <typename OUT, int NP>
 __global__ void __launch_bounds__(kPQT, 2)
     k_panel_q(PanelQ P, const long long* __restrict__ X, OUT* __restrict__ y, const WsHeader* __restrict__ h,
               unsigned long long* queue, int* err) {
@@ -271,7 +319,7 @@ __global__ void __launch_bounds__(kPQT, 2)
     const PQSmem L(P);
     int2* Ms = reinterpret_cast<int2*>(smem + L.ms);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint64_t* wl = reinterpret_cast<uint64_t*>(smem + L.lst) + warp * kPQMaxList;
+    uint64_t* wl = reinterpret_cast<uint64_t*>(smem + L.lst) + warp * 2 * kPQMaxList;
     const uint32_t dm = (1u << P.nb) - 1;
     if (h->bad) {  // an Inf or NaN in x: y is NaN and the error word is raised
         for (uint32_t pi = blockIdx.x; pi < P.npanels; pi += gridDim.x) {
@@ -291,58 +339,81 @@ __global__ void __launch_bounds__(kPQT, 2)
     __syncthreads();
     const int scale = P.emin - h->F;
     for (;;) {
-        uint32_t pi = 0;
-        if (lane == 0) pi = (uint32_t)atomicAdd(queue, 1ull);
-        pi = __shfl_sync(0xffffffffu, pi, 0);
-        if (pi >= P.npanels) break;
-        const uint32_t s0 = __ldg(P.panel_s0 + pi);
-        const uint64_t start = __ldg(P.panel_start + pi);
+        uint32_t ui = 0;
+        if (lane == 0) ui = (uint32_t)atomicAdd(queue, 1ull);
+        ui = __shfl_sync(0xffffffffu, ui, 0);
+        if (ui >= P.nunits) break;
+        const uint64_t un = __ldg(P.unit + ui);
+        uint32_t pi[NP];
+#pragma unroll
+        for (int b = 0; b < NP; ++b) pi[b] = (uint32_t)un + (b ? (uint32_t)(un >> 63) : 0u);
+        const uint32_t s0 = __ldg(P.panel_s0 + pi[0]);
         int n0 = 0;
         for (int k = 0; k < 32; k += P.nb) n0 += (int)((s0 >> k) & dm);
         const int n1 = P.N - n0;
         const int C = (int)P.t1len[n1];
-        const uint32_t hd = __ldg(P.list_hdr + pi), lo = __ldg(P.list_off + pi);
-        const int np0 = (int)(hd & 255u), nx = (int)((hd >> 8) & 255u);
-        __syncwarp();  // the warp's rows of the previous panel are done with its list slot
-        for (int q = lane; q < np0 + nx; q += 32) wl[q] = __ldg(P.list + lo + q);
+        uint64_t start[NP];
+        long long pd[NP];
+        int np0[NP], ne[NP];
+        __syncwarp();  // the warp's rows of the previous unit are done with its list slots
+#pragma unroll
+        for (int b = 0; b < NP; ++b) {
+            start[b] = __ldg(P.panel_start + pi[b]);
+            pd[b] = __ldg(P.pdiag + pi[b]);
+            const uint32_t hd = __ldg(P.list_hdr + pi[b]), lo = __ldg(P.list_off + pi[b]);
+            np0[b] = (int)(hd & 255u);
+            ne[b] = np0[b] + (int)((hd >> 8) & 255u);
+            for (int q = lane; q < ne[b]; q += 32) wl[b * kPQMaxList + q] = __ldg(P.list + lo + q);
+        }
         __syncwarp();
-        const long long pd = __ldg(P.pdiag + pi);
+        const uint32_t ch0 = (uint32_t)(un >> 32) & 0xffffu, ch1 = ch0 + ((uint32_t)(un >> 48) & 255u);
         const long long* rdg = P.rdiag + P.t1start[n1];
         const uint32_t* e1 = P.p1ell + P.p1base[n1];
-        const int m1 = (int)P.p1m[n1];
+        const unsigned char* cnt = P.p1cnt + P.p1cbase[n1];
         const uint32_t* ct = P.cutt + P.cutbase[n1];
-        const long long* Xo = X + start;
-        for (int c = lane; c < C; c += 32) {
-            const long long xo = __ldg(Xo + c);
-            const long long dg = pd + __ldg(rdg + c);
-            Acc3 a = {0, 0, 0};
+        for (uint32_t ch = ch0; ch < ch1; ++ch) {
+            const int c = (int)(ch * 32) + lane;
+            const int m1 = (int)__ldg(cnt + ch);
+            if (c >= C) continue;  // the last chunk; the warp meets again at the next unit
+            Acc3 a[NP] = {};
             // hops inside P_1: partner rows of the same panel (padding: the row itself, amplitude 0)
 #pragma unroll 4
             for (int m = 0; m < m1; ++m) {
                 const uint32_t v = __ldg(e1 + (size_t)m * C + c);
-                acc_hop(a, Ms[v >> 16], __ldg(Xo + (v & 0xffffu)));
+                const int2 am = Ms[v >> 16];
+#pragma unroll
+                for (int b = 0; b < NP; ++b) acc_hop(a[b], am, __ldg(X + start[b] + (v & 0xffffu)));
             }
-            // hops inside P_0: partner panels element by element
+#pragma unroll
+            for (int b = 0; b < NP; ++b) {
+                const uint64_t* l = wl + b * kPQMaxList;
+                // hops inside P_0: partner panels element by element
 #pragma unroll 4
-            for (int e = 0; e < np0; ++e) {
-                const uint64_t ent = wl[e];
-                acc_hop(a, Ms[ent >> 40], __ldg(X + (ent & kPQStart) + c));
-            }
-            // hops across the cut: the partner panel at the row's tabulated local index
+                for (int e = 0; e < np0[b]; ++e) {
+                    const uint64_t ent = l[e];
+                    acc_hop(a[b], Ms[ent >> 40], __ldg(X + (ent & kPQStart) + c));
+                }
+                // hops across the cut: the partner panel at the row's tabulated local index
 #pragma unroll 2
-            for (int e = np0; e < np0 + nx; ++e) {
-                const uint64_t ent = wl[e];
-                const uint32_t v = __ldg(ct + (size_t)((ent >> 40) & 255u) * C + c);
-                const int mi = (v >> 31) ? P.nM : (int)(ent >> 48) + (int)((v >> 16) & 0x7fffu);
-                acc_hop(a, Ms[mi], __ldg(X + (ent & kPQStart) + (v & 0xffffu)));
+                for (int e = np0[b]; e < ne[b]; ++e) {
+                    const uint64_t ent = l[e];
+                    const uint32_t v = __ldg(ct + (size_t)((ent >> 40) & 255u) * C + c);
+                    const int mi = (v >> 31) ? P.nM : (int)(ent >> 48) + (int)((v >> 16) & 0x7fffu);
+                    acc_hop(a[b], Ms[mi], __ldg(X + (ent & kPQStart) + (v & 0xffffu)));
+                }
             }
-            I128 r = {0, 0};
-            const long long xi = (long long)(int)(xo >> 32) * (1ll << 28) + (long long)(xo & 0xffffffffll);
-            mac(r, dg, xi);
-            add_shifted(r, a.hh, 56);
-            add_shifted(r, a.mid, 28);
-            add_shifted(r, a.ll, 0);
-            y[start + c] = i128_to<OUT>(r, scale);
+            const long long rd = __ldg(rdg + c);
+#pragma unroll
+            for (int b = 0; b < NP; ++b) {
+                const long long xo = __ldg(X + start[b] + c);
+                I128 r = {0, 0};
+                const long long xi = (long long)(int)(xo >> 32) * (1ll << 28) + (long long)(xo & 0xffffffffll);
+                mac(r, pd[b] + rd, xi);
+                add_shifted(r, a[b].hh, 56);
+                add_shifted(r, a[b].mid, 28);
+                add_shifted(r, a[b].ll, 0);
+                y[start[b] + c] = i128_to<OUT>(r, scale);
+            }
         }
     }
 }
@@ -360,14 +431,14 @@ static int run_panel_q(const dq_sector* s, const dq_terms* t, const T* x, T* y, 
     k_exp_max<T><<<sms * 8, 256, 0, st>>>(x, s->D, h);
     k_split_fixed<T><<<sms * 8, 256, 0, st>>>(x, X, s->D, h);
     const size_t sm = PQSmem(P).total;
-    auto kern = k_panel_q<T>;
+    auto kern = P.pairs ? k_panel_q<T, 2> : k_panel_q<T, 1>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return (int)e;
     int per_sm = 1;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPQT, sm)) != cudaSuccess) return (int)e;
     if (per_sm < 1) per_sm = 1;
     const uint32_t wslots = (uint32_t)sms * (uint32_t)per_sm * kPQW;
-    const unsigned grid = (unsigned)((P.npanels < wslots ? (P.npanels + kPQW - 1) / kPQW : wslots / kPQW));
+    const unsigned grid = (unsigned)((P.nunits < wslots ? (P.nunits + kPQW - 1) / kPQW : wslots / kPQW));
     const int tslot = timing_start(st);
     kern<<<grid, kPQT, sm, st>>>(P, X, y, h, queue, s->dev.err);
     timing_stop(tslot, st, 3);
