@@ -11,8 +11,9 @@
 // from those. All sums are integers, so the result does not depend on the order of the blocks.
 //
 // Before (one term after the other per row, every hop ranked, 32 terms per launch): 72 terms of the
-// 24-site disordered chain 1.0 ms in three launches plus 72 us of final sums; the figures now are at
-// k_grad_panel. Bound: integer issue, as for the product.
+// 24-site disordered chain (2.7 M rows) 1.0 ms in three launches plus 72 us of final sums. Now 167 us
+// (k_grad_panel) and 21 us (k_grad_terms), the scaling of x and dy 29 us; the differentiable step around
+// it 1.70 -> 0.76 ms. Bound: integer issue, as for the product.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
