@@ -28,15 +28,15 @@
 // the tail's particle number only; the host tabulates it (tail pattern -> local index) from the
 // sector's own rank and checks every panel's first and last row.
 //
-// Large sectors of three or more subsystems take neither: the panel kernel works on x in the order of
-// a split into TWO subsystems of its own (the "split order": P_0 = the upper L - L_1 sites, P_1 the
-// lower L_1 <= 15), whatever the sector's partition is. The prepass that makes the fixed-point copy of
-// x gathers it into that order and the kernel's stores go back through the same map. A panel of the
-// split order is a few contiguous pieces of the canonical order: the suffix bits that lie in whole
+// Large sectors whose own panels are of fewer than 15 sites take neither: the panel kernel works on x in
+// the order of a split into TWO subsystems of its own (the "split order": P_0 = the upper L - L_1 sites,
+// P_1 the lower L_1 <= 15), whatever the sector's partition is. The prepass that makes the fixed-point
+// copy of x gathers it into that order and the kernel's stores go back through the same map. A panel of
+// the split order is a few contiguous pieces of the canonical order: the suffix bits that lie in whole
 // subsystems (Llow of them) run through a contiguous range whose order depends on their particle
 // number only, one piece per pattern of the suffix bits above. One short panel per warp (k_panel_w),
 // or a tail of two short subsystems, reads about 50 partner panels per panel where 15 sites read 34.
-// 6 x 5 lattice, N = 15: three subsystems, FP32 21.4 -> 10.7 ms a product; five, FP64 23.5 -> 14.9 ms.
+// 6 x 5 lattice, N = 15: three subsystems, FP32 21.3 -> 9.5 ms a product; five, FP64 23.4 -> 13.2 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -128,18 +128,21 @@ static int build_panel_w(const dq_sector* s, PanelPlan& P, const std::vector<uin
     return DQ_OK;
 }
 
-// P_1 of the split order: the lower half of the sites, at most 15.
-static int split_sites(const dq_sector* s) { return std::min(15, s->L / 2); }
+// P_1 of the split order: as many of the lowest sites as the rank table holds (15), while at least 512
+// panels are left.
+static int split_sites(const dq_sector* s) { return std::min(15, s->L - 9); }
 
 // The split order pays for its gather of x and its scattered stores where its panels are longer than
-// those of the sector's own form (see build_panel_plan for tails of two subsystems): against warp
-// panels 1.1 to 1.6 times faster from 2 M rows on (chains of 24 to 28 sites, 4 x 6, 5 x 5 and 4 x 7
-// lattices), 2.0 times on the 6 x 5 lattice with three subsystems and FP32 vectors; against tails two
-// or more sites shorter 2.5 to 6 times, already at 0.7 M rows (22 sites, five subsystems: 0.266 ->
-// 0.059 ms). Smaller sectors keep their own form.
-static bool use_split_order(const dq_sector* s) {
+// those of the sector's own form (own_sites: P_1 of that form, 0 if it does not fit the operator), and
+// from 2^19 rows on. Each product of a panel is an own load of the partner or the rank table with little
+// else to do, so the cost of a row falls with the length of the panel: own form against split order, FP64
+// and FP32, 5 x 5 lattice (N = 12, P_1 of 12 against 15 sites) 580 -> 369, 576 -> 299 us; 9 x 3 lattice
+// (13) 2626 -> 1447, 2379 -> 1169; 7 x 4 lattice (14) 3519 -> 2946, 3048 -> 2354; chain of 24 sites (12)
+// 103 -> 90, 99 -> 80; chain of 22 sites, 0.7 M rows (11 against 13) 54 -> 47, 49 -> 43. Of equal length
+// the own form is faster (7 x 4 with P_1 of 14 sites in the split order: 3569 and 3104).
+static bool use_split_order(const dq_sector* s, int own_sites) {
     const int L1 = split_sites(s);
-    return s->n_sub >= 3 && s->D >= kSplitMinDim && s->D < (1ull << 48) && L1 > 10 && s->L - L1 <= 16;
+    return s->D >= kSplitMinDim && s->D < (1ull << 48) && L1 > 10 && L1 > own_sites && s->L - L1 <= 16;
 }
 
 // Bits of the lowest whole subsystems inside a suffix of L1 bits (L1 itself when the suffix lies
@@ -549,14 +552,15 @@ int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
     t->split = false;
     if (s->Q != 2 || s->n_sub < 2 || !uniform_lin || s->wide) return DQ_OK;
     bool fits = false;
-    if (use_split_order(s)) {
-        // the form dq_terms_path reports is the sector's own, whichever kernel runs
-        bool own = false;
-        if (int rc = build_form(s, C, pairs, t, false, true, &own)) return rc;
-        const int ns = s->n_sub, last = s->Lk[ns - 1], tail = s->Lk[ns - 2] + last;
-        const bool long_tail = own && (last < 8 || last > 10) && tail >= split_sites(s) - 1;
+    // the form dq_terms_path reports is the sector's own, whichever kernel runs
+    bool own = false;
+    if (int rc = build_form(s, C, pairs, t, false, true, &own)) return rc;
+    const int ns = s->n_sub, last = s->Lk[ns - 1];
+    const bool tail = ns >= 3 && (last < 8 || last > 10);
+    const int own_sites = !own ? 0 : tail ? s->Lk[ns - 2] + last : last;
+    if (use_split_order(s, own_sites) && (own || ns >= 3)) {
         if (int rc = build_form(s, C, pairs, t, true, true, &fits)) return rc;
-        if (fits && !long_tail) {
+        if (fits) {
             if (int rc = build_form(s, C, pairs, t, true, false, &fits)) return rc;
             if (!own) t->panel_ok = t->pw_ok = false;
             return DQ_OK;
