@@ -257,9 +257,10 @@ int dq_matvec_noalloc(const dq_sector* s, const dq_terms* t, const void* x, void
  * stored as nrhs = 2 real columns this is Re <dy, T_q x>. The gradient with respect to x is
  * H dy (every term is real and Hermitian), i.e. another dq_matvec. x, dy: device arrays laid out
  * as in dq_matvec; d_grads: device array of n_terms doubles. For Q = 2 the products dy * x are
- * exact fixed-point values (x and dy scaled per column to int64, each product rounded once to a
- * common grid with 48 bits below the largest possible product) summed in int64; other Q multiply
- * in FP64. Each block's sums are reduced in FP64 in a fixed order (deterministic). An Inf or NaN
+ * exact fixed-point values (x and dy scaled per column to int64) summed in integers: with two
+ * subsystems the sums of a thread's rows are rounded to a common grid, elsewhere each product is
+ * (48 bits below the largest possible product); other Q multiply in FP64. Repeated calls agree bit
+ * for bit. An Inf or NaN
  * in x or dy (Q = 2) gives NaN gradients and raises the sector's error word. The workspace
  * (2 * D * nrhs * 8 bytes for Q = 2, plus a few KB) is kept with the sector, grown on demand and
  * freed by dq_free_sector; calls on one sector from several host threads at once race on it.
@@ -293,9 +294,8 @@ int dq_batch_matvec(dq_batch* b, const void* const* x, void* const* y, void* str
 /* Autotuner: time every candidate (row mapping, threads per CTA, CTAs per SM, rows per tile) on
  * the given vectors (one warm-up and three timed launches each, CUDA events on `stream`), keep
  * the fastest for later dq_batch_matvec calls and return its number in *choice (may be NULL).
- * The mappings: the CTA's threads take a tile's rows with a block stride and unrank each with
- * Alg. 4, or each warp takes 32 R consecutive rows and each lane steps from row to row through
- * the last subsystem's unrank list. Tiles are pulled from an atomic queue in both. Overwrites y.
+ * The mappings: a warp unranks each of its rows with Alg. 4, or each lane steps from row to row
+ * through the last subsystem's unrank list. Tiles are pulled from an atomic queue in both. Overwrites y.
  * Synchronous. */
 int dq_batch_tune(dq_batch* b, const void* const* x, void* const* y, void* stream, int* choice);
 
