@@ -179,9 +179,10 @@ int dq_make_terms(const dq_sector* s, const dq_term* terms, int n_terms, dq_term
  * (Nbits * L_1 <= 14) and P_0 of at most 24, no n_i n_j pair terms, D < 2^40, at most 31 hop
  * bonds and 4096 hop amplitude entries (bonds x Q x Q), 64 P_0 and cut hops per panel; any
  * coefficient per hop bond and any site function (the per-term form's integer coefficients, so
- * it gives the general kernel's y). With three or more subsystems the value names the form that fits
- * the sector's own partition; sectors of at least 2^19 rows whose operator fits two halves of the
- * lattice run the panel kernel on those halves instead, with the same y. */
+ * it gives the general kernel's y). The values 0, 1 and 4 name the form that fits the sector's own
+ * partition; sectors of at least 2^19 rows whose own panels are of fewer than 15 sites run the panel
+ * kernel on the lowest 15 sites (L - 9 below 24 sites) instead where the operator fits it, with the
+ * same y. */
 int dq_terms_path(const dq_terms* t, int* path);
 
 /* Compile terms in the cluster-merged form of App. C instead: the terms are grouped into clusters
@@ -262,7 +263,8 @@ int dq_matvec_noalloc(const dq_sector* s, const dq_terms* t, const void* x, void
  * (48 bits below the largest possible product); other Q multiply in FP64. Repeated calls agree bit
  * for bit. An Inf or NaN
  * in x or dy (Q = 2) gives NaN gradients and raises the sector's error word. The workspace
- * (2 * D * nrhs * 8 bytes for Q = 2, plus a few KB) is kept with the sector, grown on demand and
+ * (2 * D * nrhs * 8 bytes for Q = 2, plus the sums: a few KB, or some 8-byte words per panel and per
+ * P_1 pattern) is kept with the sector, grown on demand and
  * freed by dq_free_sector; calls on one sector from several host threads at once race on it.
  * Synchronous. Errors as dq_make_terms, plus DQ_EINVAL for bad dtype or nrhs or a sector of
  * two-word states, DQ_ENOMEM. The paper's operator class (Sec. 4.1) has no derivatives; this
