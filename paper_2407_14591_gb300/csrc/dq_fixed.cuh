@@ -170,6 +170,23 @@ __device__ __forceinline__ void add_shifted(I128& a, long long v, int sh) {
     a.lo = s;
 }
 
+// A sum of many |X| <= 2^56 in two words, top 2^48 + low: fold_sum moves what is above 48 bits of the low
+// word into the top one (at most 64 terms between two folds, so the low word stays below 2^63), add_folded
+// adds m times the sum to r.
+constexpr int kFoldBits = 48;
+__device__ __forceinline__ void fold_sum(long long& low, int& top) {
+    top += (int)(low >> kFoldBits);
+    low &= (1ll << kFoldBits) - 1;
+}
+__device__ __forceinline__ void add_folded(I128& r, long long m, long long low, int top) {
+    mac(r, m, low);
+    I128 t = {0, 0};
+    mac(t, m, top);
+    const unsigned long long lo = t.lo << kFoldBits, s = r.lo + lo;
+    r.hi += (long long)(((unsigned long long)t.hi << kFoldBits) | (t.lo >> (64 - kFoldBits))) + (s < r.lo ? 1 : 0);
+    r.lo = s;
+}
+
 // ------------------------------------------------------------------ per-column prepass -------
 
 // Scales of an interleaved block of nrhs <= 64 columns (x[i * nrhs + c]).

@@ -112,6 +112,7 @@ constexpr int kPanelMaxLayers = 16;
 constexpr int kPanelMaxGroups = 16;
 constexpr int kPanelMaxA = 2;  // distinct hop amplitudes
 constexpr int kPanelMaxK = 4;  // distinct [s_i != s_j] coefficients
+constexpr int kPanelMaxHops = 127;  // 2^56 each: an int64 sum stays below 2^63
 constexpr int kPanelMaxList = kPanelMaxBonds + kPanelMaxGroups;
 // Per-panel values shared by all rows of the panel: counts of [s_i != s_j] over the Sz Sz bonds
 // inside P_0 per coefficient class, and the bit-plane counters (3 bits per position b of P_1) of
@@ -161,6 +162,9 @@ struct PanelPlan {
     long long MC, MK[kPanelMaxK], MA[kPanelMaxA];  // coefficients / 2^emin
     int emin;
     int cmax;  // longest panel
+    // float64 vectors: a row can have more hops of one amplitude than an int64 holds of |X| <= 2^56
+    // (kPanelMaxHops), so the kernels fold their sums on the way
+    bool fold;
     // per-panel source lists (built on the host): panel p owns entries [list_off[p], list_off[p+1])
     // = its active P_0 partners (first list_cnt0[p] of class 0, then class 1) and then its valid
     // crossing partners. Entry: global start index | (crossing group << 48).

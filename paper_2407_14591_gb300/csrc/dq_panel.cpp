@@ -154,6 +154,27 @@ static int whole_bits(const dq_sector* s, int L1) {
     return low;
 }
 
+// Most hops of one amplitude class that a row can have, as a bound: of the bonds between two groups of
+// sites those between an occupied and an empty one hop.
+static int most_hops(const PanelPlan& P, const std::vector<std::pair<int, uint32_t>>& p0,
+                     const std::map<int, std::vector<std::pair<int, int>>>& p1,
+                     const std::map<uint32_t, std::vector<std::pair<int, uint32_t>>>& cut) {
+    int most = 0;
+    for (int k = 0; k < kPanelMaxA; ++k) {
+        int b0 = 0, b1 = 0, bx = 0;
+        for (auto& e : p0) b0 += e.first == k;
+        for (auto& g : p1)
+            for (auto& e : g.second) b1 += e.first == k;
+        for (auto& g : cut)
+            for (auto& e : g.second) bx += e.first == k;
+        for (int n0 = std::max(0, P.N - P.L1); n0 <= std::min(P.L0, P.N); ++n0) {
+            const int n1 = P.N - n0, e0 = P.L0 - n0, e1 = P.L1 - n1;
+            most = std::max(most, std::min(b0, n0 * e0) + std::min(b1, n1 * e1) + std::min(bx, n0 * e1 + n1 * e0));
+        }
+    }
+    return most;
+}
+
 // One form of the plan: the sector's own order or the split order. *fits: the operator's bonds and
 // coefficients fit the form; with check_only nothing else is done.
 static int build_form(const dq_sector* s, double C,
@@ -317,6 +338,7 @@ static int build_form(const dq_sector* s, double C,
     for (int k = 0; k < P.nA; ++k)
         if (!scaled(Avals[k], P.MA[k])) return DQ_OK;
     P.emin = emin;
+    P.fold = most_hops(P, p0o, p1o, xo) > kPanelMaxHops;
     *fits = true;
     if (check_only) return DQ_OK;
     // P_1 tables (local index within its particle-number sector, and the states per sector)

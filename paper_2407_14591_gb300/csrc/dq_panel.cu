@@ -28,7 +28,7 @@ int launch_panel_matvec_ws(const dq_sector* s, const dq_terms* t, const void* x,
     cudaStream_t st = (cudaStream_t)stream;
     const int na = t->pp.nA;
     if (dtype == DQ_F64) {
-        if (na <= 1) return run_panel_n<double, long long, 1>(s, t, (const double*)x, (double*)y, ws, st);
+        if (na <= 1 && !t->pp.fold) return run_panel_n<double, long long, 1>(s, t, (const double*)x, (double*)y, ws, st);
         return run_panel_n<double, long long, 2>(s, t, (const double*)x, (double*)y, ws, st);
     }
     if (na <= 1) return run_panel_n<float, int, 1>(s, t, (const float*)x, (float*)y, ws, st);

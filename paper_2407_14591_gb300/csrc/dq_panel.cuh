@@ -5,7 +5,8 @@
 // are exact integer sums: a prepass scales x by 2^F (F from the largest exponent in x) and
 // rounds it to int64 (FP64 input, |X| < 2^56) or int32 (FP32 input, |X| < 2^30); every hop adds
 // an integer; the row result sum_k M_k T_k (coefficients M_k = c_k / 2^emin, integers) is formed
-// in 128-bit integers and rounded once to the output type. The only error is the rounding of
+// in 128-bit integers and rounded once to the output type (operators that can have more than 127 hops
+// of one amplitude in a row run a variant that folds T_k into two words). The only error is the rounding of
 // x to 2^-F, at most 2^-57 (FP64) or 2^-31 (FP32) of max|x| per term.
 //
 // Data movement. One CTA per panel (all rows with one P_0 pattern s0, contiguous in the
@@ -176,7 +177,7 @@ __device__ __forceinline__ void release_slot(int s, int jn, const PanelPlan& P, 
 
 // All the work of one panel for rows tid + e * NT, e < E. Rows past the panel hold s = 0: their
 // gathers read in-range entries, and they are never stored.
-template <typename XT, typename OUT, int NA, int R, int E, int NT, bool SPLIT>
+template <typename XT, typename OUT, int NA, int R, int E, int NT, bool SPLIT, bool FOLD>
 __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restrict__ X, OUT* __restrict__ y,
                                            unsigned char* smem, uint64_t* bar, const uint64_t* lst, const long long* sums,
                                            const PanelCtx& pc, size_t bstride, uint32_t& ph, int scale, int& fail,
@@ -185,13 +186,17 @@ __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restr
     const unsigned char* own = smem + kOwn;
     uint32_t s2[E];  // P_1 pattern of each row, shifted left by one (rank-table byte offset)
     long long acc[NA][E];
+    int top[FOLD ? NA : 1][FOLD ? E : 1];
     const uint16_t* st = P.t1states + P.t1start[pc.n1];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         int c = tid + e * NT;
         s2[e] = c < pc.C ? ((uint32_t)__ldg(st + c) << 1) : 0u;
 #pragma unroll
-        for (int k = 0; k < NA; ++k) acc[k][e] = 0;
+        for (int k = 0; k < NA; ++k) {
+            acc[k][e] = 0;
+            if constexpr (FOLD) top[k][e] = 0;
+        }
     }
     // The work of the panel in units that need no copy: P_0 partner panels two at a time (per
     // amplitude class), and P_1 bond layers. They are interleaved with the cross partners of
@@ -270,9 +275,21 @@ __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restr
             }
         }
     };
+    // after every unit and every cut partner: at most 64 hops of one amplitude
+    auto fold = [&]() {
+        if constexpr (FOLD) {
+#pragma unroll
+            for (int k = 0; k < NA; ++k)
+#pragma unroll
+                for (int e = 0; e < E; ++e) fold_sum(acc[k][e], top[k][e]);
+        }
+    };
     int u = 0;
     const int lead = pc.nx ? (nu < 2 ? nu : 2) : nu;  // units before the first cross partner
-    for (; u < lead; ++u) run_unit(u);
+    for (; u < lead; ++u) {
+        run_unit(u);
+        fold();
+    }
     int target = lead, frac = 0;
     // hops across the cut: panel s0 ^ bit_a of the neighbouring block, in the copy ring
     for (int j = 0; j < pc.nx; ++j) {
@@ -298,6 +315,7 @@ __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restr
                 }
             }
         }
+        fold();
         release_slot<XT, R, NT>(s, j + R - 1, P, pc, X, smem, bstride, bar, lst, rg);
         // target = lead + floor((nu - lead) (j + 1) / nx), kept incrementally
         frac += nu - lead;
@@ -305,9 +323,15 @@ __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restr
             frac -= pc.nx;
             ++target;
         }
-        for (; u < target; ++u) run_unit(u);
+        for (; u < target; ++u) {
+            run_unit(u);
+            fold();
+        }
     }
-    for (; u < nu; ++u) run_unit(u);
+    for (; u < nu; ++u) {
+        run_unit(u);
+        fold();
+    }
     // the row result: (diagonal) x_i + sum_k A_k S_k, exactly, rounded once. The diagonal is the
     // pattern's P_1 Sz Sz sum (a table) and the panel's two sums (its constant and the cut bonds)
     // (6 x 5 lattice, N = 15: counting the bonds per row took 0.7 ms of 13.3 in FP64, 0.9 of 10.0 in FP32)
@@ -321,7 +345,12 @@ __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restr
         I128 r = {0, 0};
         mac(r, md, lds_x<XT>(own, (uint32_t)(c * sizeof(XT))));
 #pragma unroll
-        for (int k = 0; k < NA; ++k) mac(r, P.MA[k], acc[k][e]);
+        for (int k = 0; k < NA; ++k) {
+            if constexpr (FOLD)
+                add_folded(r, P.MA[k], acc[k][e], top[k][e]);
+            else
+                mac(r, P.MA[k], acc[k][e]);
+        }
         uint64_t to = pc.start + c;
         if constexpr (SPLIT) {
             const uint32_t yo = __ldg(P.rowy + P.t1start[pc.n1] + c);
@@ -331,7 +360,7 @@ __device__ __forceinline__ void panel_rows(const PanelPlan& P, const XT* __restr
     }
 }
 
-template <typename XT, typename OUT, int NA, int R, int NT, bool SPLIT>
+template <typename XT, typename OUT, int NA, int R, int NT, bool SPLIT, bool FOLD>
 __global__ void __launch_bounds__(NT, kPT / NT)
     k_panel(PanelPlan P, const XT* __restrict__ X, OUT* __restrict__ y, const WsHeader* __restrict__ h, int* err,
             int cap) {
@@ -432,19 +461,19 @@ __global__ void __launch_bounds__(NT, kPT / NT)
         // 1024 threads; 512-thread CTAs take panels of at most 1024 rows)
         if constexpr (NT == kPT) {
             switch ((pc.C + NT - 1) / NT) {
-                case 7: panel_rows<XT, OUT, NA, R, 7, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
-                case 6: panel_rows<XT, OUT, NA, R, 6, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
-                case 5: panel_rows<XT, OUT, NA, R, 5, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
-                case 4: panel_rows<XT, OUT, NA, R, 4, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
-                case 3: panel_rows<XT, OUT, NA, R, 3, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
-                case 2: panel_rows<XT, OUT, NA, R, 2, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
-                default: panel_rows<XT, OUT, NA, R, 1, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
+                case 7: panel_rows<XT, OUT, NA, R, 7, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 6: panel_rows<XT, OUT, NA, R, 6, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 5: panel_rows<XT, OUT, NA, R, 5, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 4: panel_rows<XT, OUT, NA, R, 4, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 3: panel_rows<XT, OUT, NA, R, 3, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                case 2: panel_rows<XT, OUT, NA, R, 2, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg); break;
+                default: panel_rows<XT, OUT, NA, R, 1, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
             }
         } else {
             if (pc.C > NT)
-                panel_rows<XT, OUT, NA, R, 2, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
+                panel_rows<XT, OUT, NA, R, 2, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
             else
-                panel_rows<XT, OUT, NA, R, 1, NT, SPLIT>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
+                panel_rows<XT, OUT, NA, R, 1, NT, SPLIT, FOLD>(P, X, y, smem, bar, lst, sums, pc, bstride, ph, scale, fail, rg);
         }
     }
     if (fail) s_fail = 1;
@@ -485,7 +514,7 @@ __global__ void __launch_bounds__(256) k_to_fixed_split(PanelPlan P, const T* __
     }
 }
 
-template <typename T, typename XT, int NA, int R, int NT, bool SPLIT>
+template <typename T, typename XT, int NA, int R, int NT, bool SPLIT, bool FOLD = false>
 static int run_panel(const dq_sector* s, const dq_terms* t, const T* x, T* y, void* ws, cudaStream_t st) {
     const PanelPlan& P = t->pp;
     WsHeader* h = reinterpret_cast<WsHeader*>(ws);
@@ -499,7 +528,7 @@ static int run_panel(const dq_sector* s, const dq_terms* t, const T* x, T* y, vo
         k_to_fixed<T, XT><<<sms * 8, 256, 0, st>>>(x, X, s->D, h);
     const int cap = P.cmax + 16 / (int)sizeof(XT) + 4;
     size_t sm = PanelSmem<XT>::total(cap, R);
-    auto kern = k_panel<XT, T, NA, R, NT, SPLIT>;
+    auto kern = k_panel<XT, T, NA, R, NT, SPLIT, FOLD>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return (int)e;
     int per_sm = 1;
@@ -515,6 +544,9 @@ static int run_panel(const dq_sector* s, const dq_terms* t, const T* x, T* y, vo
 
 template <typename T, typename XT, int NA, bool SPLIT>
 int run_panel_s(const dq_sector* s, const dq_terms* t, const T* x, T* y, void* ws, cudaStream_t st) {
+    // rare operators: one variant for every panel length and both numbers of amplitudes
+    if constexpr (sizeof(XT) == 8 && NA == kPanelMaxA)
+        if (t->pp.fold) return run_panel<T, XT, NA, 3, kPT, SPLIT, true>(s, t, x, y, ws, st);
     // copy slots (the panel's own buffer and the staging buffers) that fit next to the rank
     // table in 227 KB of shared memory; panels of at most 1024 rows run two 512-thread CTAs per
     // SM, with six slots when two such CTAs still fit in one SM's shared memory

@@ -160,7 +160,7 @@ __device__ __forceinline__ void pw_setup(const PanelPlan& P, const PWRank& R, co
 }
 
 // The rows of one panel, rows lane + 32 e (e < E) of the warp.
-template <typename XT, typename OUT, int NA, int E>
+template <typename XT, typename OUT, int NA, int E, bool FOLD>
 __device__ __forceinline__ void pw_rows(const PanelPlan& P, const XT* __restrict__ X, OUT* __restrict__ y,
                                         const unsigned char* tab, const unsigned char* own, unsigned char* slot,
                                         const uint64_t* lst, const PanelDiag* dg, const PWPanel& pp, int scale) {
@@ -168,14 +168,27 @@ __device__ __forceinline__ void pw_rows(const PanelPlan& P, const XT* __restrict
     const int C = pp.C;
     uint32_t s2[E];  // P_1 pattern of each row, shifted left by one (rank-table byte offset)
     long long acc[NA][E];
+    int top[FOLD ? NA : 1][FOLD ? E : 1];
     const uint16_t* st = P.t1states + P.t1start[pp.n1];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int c = lane + 32 * e;
         s2[e] = c < C ? ((uint32_t)__ldg(st + c) << 1) : 0u;
 #pragma unroll
-        for (int k = 0; k < NA; ++k) acc[k][e] = 0;
+        for (int k = 0; k < NA; ++k) {
+            acc[k][e] = 0;
+            if constexpr (FOLD) top[k][e] = 0;
+        }
     }
+    // after the hops of each place and after every cut partner: at most 64 of one amplitude
+    auto fold = [&]() {
+        if constexpr (FOLD) {
+#pragma unroll
+            for (int k = 0; k < NA; ++k)
+#pragma unroll
+                for (int e = 0; e < E; ++e) fold_sum(acc[k][e], top[k][e]);
+        }
+    };
     // hops inside P_0: partner panels element by element, by amplitude class (two partners per
     // round with int32 elements; int64 elements would need more registers than four CTAs per SM
     // leave)
@@ -194,6 +207,7 @@ __device__ __forceinline__ void pw_rows(const PanelPlan& P, const XT* __restrict
                 }
             }
     }
+    fold();
     // hops inside P_1, one bond layer of distance d at a time
     for (int ly = 0; ly < P.n_p1l; ++ly) {
         const int d = P.p1l_d[ly];
@@ -210,6 +224,7 @@ __device__ __forceinline__ void pw_rows(const PanelPlan& P, const XT* __restrict
             }
         }
     }
+    fold();
     // hops across the cut: the partner panel s0 ^ bit_a staged in the warp's second slot
     const int np0 = pp.np0[0] + (NA > 1 ? pp.np0[NA - 1] : 0);
     for (int g = 0; g < P.n_xg; ++g) {
@@ -235,6 +250,7 @@ __device__ __forceinline__ void pw_rows(const PanelPlan& P, const XT* __restrict
                 }
             }
         }
+        fold();
     }
     // the row result: (C + sum_k K_k n_k) x_i + sum_k A_k S_k, exactly, rounded once
     const uint32_t m1 = (1u << P.L1) - 1u;
@@ -257,13 +273,18 @@ __device__ __forceinline__ void pw_rows(const PanelPlan& P, const XT* __restrict
         I128 r = {0, 0};
         mac(r, md, pw_lds<XT>(own, (uint32_t)(c * sizeof(XT))));
 #pragma unroll
-        for (int k = 0; k < NA; ++k) mac(r, P.MA[k], acc[k][e]);
+        for (int k = 0; k < NA; ++k) {
+            if constexpr (FOLD)
+                add_folded(r, P.MA[k], acc[k][e], top[k][e]);
+            else
+                mac(r, P.MA[k], acc[k][e]);
+        }
         y[pp.start + c] = i128_to<OUT>(r, scale);
     }
 }
 
 // Four CTAs (32 warps) per SM: at most 64 registers per thread.
-template <typename XT, typename OUT, int NA>
+template <typename XT, typename OUT, int NA, bool FOLD>
 __global__ void __launch_bounds__(kPWT, 4) k_panel_w(PanelPlan P, PWRank R, const XT* __restrict__ X, OUT* __restrict__ y,
                                                   const WsHeader* __restrict__ h, int* err) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -311,20 +332,20 @@ __global__ void __launch_bounds__(kPWT, 4) k_panel_w(PanelPlan P, PWRank R, cons
         pw_setup(P, R, off_s, str_s, lst, dg, pp, err);
         __syncwarp();
         switch ((pp.C + 31) >> 5) {
-            case 8: pw_rows<XT, OUT, NA, 8>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
-            case 7: pw_rows<XT, OUT, NA, 7>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
-            case 6: pw_rows<XT, OUT, NA, 6>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
-            case 5: pw_rows<XT, OUT, NA, 5>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
-            case 4: pw_rows<XT, OUT, NA, 4>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
-            case 3: pw_rows<XT, OUT, NA, 3>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
-            case 2: pw_rows<XT, OUT, NA, 2>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
-            default: pw_rows<XT, OUT, NA, 1>(P, X, y, smem, own, slot, lst, dg, pp, scale);
+            case 8: pw_rows<XT, OUT, NA, 8, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
+            case 7: pw_rows<XT, OUT, NA, 7, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
+            case 6: pw_rows<XT, OUT, NA, 6, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
+            case 5: pw_rows<XT, OUT, NA, 5, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
+            case 4: pw_rows<XT, OUT, NA, 4, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
+            case 3: pw_rows<XT, OUT, NA, 3, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
+            case 2: pw_rows<XT, OUT, NA, 2, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale); break;
+            default: pw_rows<XT, OUT, NA, 1, FOLD>(P, X, y, smem, own, slot, lst, dg, pp, scale);
         }
     }
 }
 
 // ws: the fixed-point scratch (header and X, panel_scratch_bytes).
-template <typename T, typename XT, int NA>
+template <typename T, typename XT, int NA, bool FOLD = false>
 static int run_pw(const dq_sector* s, const dq_terms* t, const T* x, T* y, void* ws, cudaStream_t st) {
     const PanelPlan& P = t->pp;
     WsHeader* h = reinterpret_cast<WsHeader*>(ws);
@@ -334,7 +355,7 @@ static int run_pw(const dq_sector* s, const dq_terms* t, const T* x, T* y, void*
     k_exp_max<T><<<sms * 8, 256, 0, st>>>(x, s->D, h);
     k_to_fixed<T, XT><<<sms * 8, 256, 0, st>>>(x, X, s->D, h);
     const size_t sm = PWSmem<XT>::total(t->pwr.os_total);
-    auto kern = k_panel_w<XT, T, NA>;
+    auto kern = k_panel_w<XT, T, NA, FOLD>;
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return (int)e;
@@ -353,6 +374,8 @@ int launch_panel_w_ws(const dq_sector* s, const dq_terms* t, const void* x, void
                       void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     const bool two = t->pp.nA > 1;
+    if (dtype == DQ_F64 && t->pp.fold)
+        return run_pw<double, long long, 2, true>(s, t, (const double*)x, (double*)y, ws, st);
     if (dtype == DQ_F64)
         return two ? run_pw<double, long long, 2>(s, t, (const double*)x, (double*)y, ws, st)
                    : run_pw<double, long long, 1>(s, t, (const double*)x, (double*)y, ws, st);
