@@ -258,10 +258,10 @@ int dq_matvec_noalloc(const dq_sector* s, const dq_terms* t, const void* x, void
  * stored as nrhs = 2 real columns this is Re <dy, T_q x>. The gradient with respect to x is
  * H dy (every term is real and Hermitian), i.e. another dq_matvec. x, dy: device arrays laid out
  * as in dq_matvec; d_grads: device array of n_terms doubles. For Q = 2 the products dy * x are
- * exact fixed-point values (x and dy scaled per column to int64) summed in integers: with two
- * subsystems the sums of a thread's rows are rounded to a common grid, elsewhere each product is
- * (48 bits below the largest possible product); other Q multiply in FP64. Repeated calls agree bit
- * for bit. An Inf or NaN
+ * exact fixed-point values (x and dy scaled per column to int64) summed in integers on a common
+ * grid, 48 bits below the largest possible sum of a row's products over the columns: every product
+ * is rounded to it once or, with two subsystems, the sum of a few rows' products is. Other Q
+ * multiply in FP64. Repeated calls agree bit for bit. An Inf or NaN
  * in x or dy (Q = 2) gives NaN gradients and raises the sector's error word. The workspace
  * (2 * D * nrhs * 8 bytes for Q = 2, plus the sums: a few KB, or some 8-byte words per panel and per
  * P_1 pattern) is kept with the sector, grown on demand and

@@ -6,9 +6,11 @@
 // P_1 and across the cut with an element of the panel or of the panel s0 ^ bit_a through a rank table in
 // shared memory. Per panel and hop pair each thread sums its rows' dy * x in 64-bit integers (x and dy
 // split in 32-bit halves), rounds the sum once onto a common grid 2^-G and a warp adds it to its own
-// accumulator. The diagonal terms need only p_i = dy_i x_i: its sum per panel (P_0 terms), per P_1
-// pattern (P_1 terms), and per panel and P_1 bit (pairs across the cut); a last kernel forms every term
-// from those. All sums are integers, so the result does not depend on the order of the blocks.
+// accumulator. The diagonal terms need only p_i = dy_i x_i, rounded one by one: its sum per panel (P_0
+// terms), per P_1 pattern (P_1 terms), and per panel and P_1 bit (pairs across the cut); a last kernel
+// forms every term from those. All sums are integers, so the result does not depend on the order of the
+// blocks. A block empties its accumulators into the two-word totals before one of them can fill, so the
+// grid keeps 48 bits, shared out over the columns, for any number of panels and columns.
 //
 // Before (one term after the other per row, every hop ranked, 32 terms per launch): 72 terms of the
 // 24-site disordered chain (2.7 M rows) 1.0 ms in three launches plus 72 us of final sums. Now 167 us
@@ -33,7 +35,9 @@ constexpr int kGPW = kGPT / 32;
 constexpr int kGPSlots = 2;      // cut partner panels held at a time
 constexpr int kGPPairs = 64;     // hop pairs of one place (P_0, P_1, cut); pairs of the cut with a diagonal
 constexpr int kGPGroups = 16;
-constexpr int kGPBits = 48;      // |dy x| on the grid, before the columns are added
+constexpr int kGPBits = 48;      // |dy x| on the grid, summed over the columns
+// rows of one column that a warp or a P_1 pattern may add up before its sum is emptied: below 2^62
+constexpr uint64_t kGPRows = 1ull << (62 - kGPBits);
 
 struct GradPlan {
     int L0, L1, N, cap, npair;
@@ -236,19 +240,19 @@ __device__ __forceinline__ void grad_rows(const GradPlan& P, const GradSmem& L, 
     }
 }
 
-__device__ __forceinline__ void grad_scales(const ColScale* hx, const ColScale* hdy, int cols, int bits, int* G, int* sh) {
-    // common grid: the largest column bound of |dy x| lands below 2^(bits - lg cols)
+__device__ __forceinline__ void grad_scales(const ColScale* hx, const ColScale* hdy, int cols, int* G, int* sh) {
+    // common grid: the largest column bound of |dy x| lands below 2^(kGPBits - lg cols)
     int lg = 0;
     while ((1 << lg) < cols) ++lg;
     int fmin = 1 << 30;
     for (int r = 0; r < cols; ++r) fmin = min(fmin, hx->F[r] + hdy->F[r]);
-    *G = fmin - (112 - bits) - lg;  // |X| and |DY| stay below 2^56
+    *G = fmin - (112 - kGPBits) - lg;  // |X| and |DY| stay below 2^56
     for (int r = 0; sh && r < cols; ++r) sh[r] = hx->F[r] + hdy->F[r] - *G;
 }
 
 __global__ void __launch_bounds__(kGPT, 2)
     k_grad_panel(GradPlan P, GradSmem L, const long long* __restrict__ X, const long long* __restrict__ DY,
-                 const ColScale* __restrict__ hx, const ColScale* __restrict__ hdy, uint64_t xstride, int cols, int bits,
+                 const ColScale* __restrict__ hx, const ColScale* __restrict__ hdy, uint64_t xstride, int cols, int period,
                  GradSums out) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int sh_s[kMaxCols], G_s;
@@ -262,8 +266,29 @@ __global__ void __launch_bounds__(kGPT, 2)
         reinterpret_cast<long long*>(smem + L.own + (q / 8) * L.bstride)[P.cap + q % 8] = 0;
     for (uint32_t q = tid; q < ntab; q += kGPT) reinterpret_cast<long long*>(smem + L.W)[q] = 0;
     for (int q = tid; q < kGPW * P.npair; q += kGPT) reinterpret_cast<long long*>(smem + L.acc)[q] = 0;
-    if (tid == 0) grad_scales(hx, hdy, cols, bits, &G_s, sh_s);
+    if (tid == 0) grad_scales(hx, hdy, cols, &G_s, sh_s);
+    // the block's sums into the totals, and from zero again (between two barriers)
+    auto empty = [&]() {
+        for (uint32_t q = tid; q < ntab; q += kGPT) {
+            long long& v = reinterpret_cast<long long*>(smem + L.W)[q];
+            if (v) grad_red(out.Wlo + q, out.Whi + q, v);
+            v = 0;
+        }
+        for (int q = tid; q < P.npair; q += kGPT) {
+            long long hi = 0;  // a warp's sums stay below 2^62, eight of them below 2^65
+            unsigned long long lo = 0;
+            for (int w = 0; w < kGPW; ++w) {
+                long long& a = reinterpret_cast<long long*>(smem + L.acc)[w * P.npair + q];
+                lo += (unsigned long long)(a & 0xffffffffll);
+                hi += a >> 32;
+                a = 0;
+            }
+            atomicAdd(out.Alo + q, lo);
+            atomicAdd(out.Ahi + q, (unsigned long long)hi);
+        }
+    };
     const uint64_t items = (uint64_t)P.npanels * cols;
+    int since = 0;  // items since the sums were last emptied
     for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
         const uint32_t pi = (uint32_t)(item / cols);
         const int col = (int)(item % cols);
@@ -272,6 +297,12 @@ __global__ void __launch_bounds__(kGPT, 2)
         const int n1 = P.N - __popc(s0), C = (int)P.t1len[n1];
         const long long* Xc = X + col * xstride;
         __syncthreads();  // the previous panel is finished
+        if (since == period) {
+            empty();
+            __syncthreads();  // a warp's own rows begin with its accumulators
+            since = 0;
+        }
+        ++since;
         long long* own = reinterpret_cast<long long*>(smem + L.own);
         for (int c = tid; c < C; c += kGPT) grad_copy(own + c, Xc + start + c);
         for (int j = 0; j < kGPSlots && j < P.nxg; ++j) {
@@ -295,27 +326,13 @@ __global__ void __launch_bounds__(kGPT, 2)
 #undef GRAD_ROWS
     }
     __syncthreads();
-    for (uint32_t q = tid; q < ntab; q += kGPT) {
-        const long long v = reinterpret_cast<const long long*>(smem + L.W)[q];
-        if (v) grad_red(out.Wlo + q, out.Whi + q, v);
-    }
-    for (int q = tid; q < P.npair; q += kGPT) {
-        long long v = 0;  // a warp's sums stay below 2^62 (the host's choice of bits), eight of them below 2^65
-        unsigned long long lo = 0;
-        for (int w = 0; w < kGPW; ++w) {
-            const long long a = reinterpret_cast<const long long*>(smem + L.acc)[w * P.npair + q];
-            lo += (unsigned long long)(a & 0xffffffffll);
-            v += a >> 32;
-        }
-        atomicAdd(out.Alo + q, lo);
-        atomicAdd(out.Ahi + q, (unsigned long long)v);
-    }
+    empty();
 }
 
 // Output q, one block each: f * sum of sign * p in units of 2^-G.
 __global__ void __launch_bounds__(256)
     k_grad_terms(GradPlan P, GradSums in, const GradOut* __restrict__ outs, const ColScale* __restrict__ hx,
-                 const ColScale* __restrict__ hdy, int cols, int bits, double* __restrict__ g, int* err) {
+                 const ColScale* __restrict__ hdy, int cols, double* __restrict__ g, int* err) {
     __shared__ long long red[2][8];
     const GradOut o = outs[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -379,7 +396,7 @@ __global__ void __launch_bounds__(256)
             g[blockIdx.x] = __longlong_as_double(0x7ff8000000000000ll);
             if (blockIdx.x == 0) atomicAdd(err, 1);
         } else {
-            grad_scales(hx, hdy, cols, bits, &G, nullptr);
+            grad_scales(hx, hdy, cols, &G, nullptr);
             g[blockIdx.x] = ldexp(f * ((double)hi * 4294967296.0 + (double)lo), -G);
         }
     }
@@ -547,11 +564,9 @@ int launch_grad_panel(const dq_sector* s, const dq_term* terms, int n_terms, con
     const int per_sm = occupancy_cached(reinterpret_cast<const void*>(kern), kGPT, L.total);
     const uint64_t items = (uint64_t)P.npanels * cols;
     const unsigned grid = (unsigned)std::min<uint64_t>(std::max<uint64_t>(items, 1), (uint64_t)sms * per_sm);
-    // grid of the products: a warp's sum of one pair (its rows of all its panels) stays below 2^62
-    const uint64_t rows = (items + grid - 1) / grid * (uint64_t)((P.cap + kGPT - 1) / kGPT) * 32;
-    int lg = 0;
-    while ((1ull << lg) < rows) ++lg;
-    const int bits = std::min(kGPBits, 62 - lg);
+    // items of a block between two emptyings: a warp takes up to this many rows of a panel
+    const uint64_t rows = (uint64_t)((P.cap + kGPT - 1) / kGPT) * 32;
+    const int period = (int)(kGPRows / rows);
     // workspace: the two scales and the sums (zeroed), the outputs, the copies of x and dy
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const uint64_t xstride = (s->D + 15) & ~15ull;
@@ -585,8 +600,8 @@ int launch_grad_panel(const dq_sector* s, const dq_term* terms, int n_terms, con
         k_grad_exp_max<float><<<pgrid, bs, 0, st>>>((const float*)x, (const float*)dy, n, cols, hx, hdy);
         k_grad_fixed<float><<<pgrid, bs, 0, st>>>((const float*)x, (const float*)dy, X, DY, n, cols, xstride, hx, hdy);
     }
-    kern<<<grid, kGPT, L.total, st>>>(P, L, X, DY, hx, hdy, xstride, cols, bits, sum);
-    k_grad_terms<<<n_terms, 256, 0, st>>>(P, sum, d_out, hx, hdy, cols, bits, d_grads, s->dev.err);
+    kern<<<grid, kGPT, L.total, st>>>(P, L, X, DY, hx, hdy, xstride, cols, period, sum);
+    k_grad_terms<<<n_terms, 256, 0, st>>>(P, sum, d_out, hx, hdy, cols, d_grads, s->dev.err);
     timing_stop(tslot, st, 4);
     return (int)cudaGetLastError();
 }
