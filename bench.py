@@ -47,6 +47,10 @@ NCU_TRAFFIC = {
     ("j1j2_square_6x5_N15", 2, "f32", 1, "817aac068746ea5d"): 6.956715776e9,
 }
 
+# kernel names by the binding's name of the kernel a product runs; the others are the general kernels
+KERNELS = {"panel": "k_panel", "panel_split": "k_panel", "panel_pb": "k_panel_pb", "panel_w": "k_panel_w",
+           "panel_q": "k_panel_q", "cluster": "k_matvec_cl"}
+
 WORKLOADS = {
     "j1j2": 2,
     "chain": 1,
@@ -466,9 +470,9 @@ def run_diff(args, world, rank, local, dist, torch):
                        "step": "y = H(theta) x, then dx and dtheta"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": None, "peak_source": peak_kind, "algorithmic_bytes_per_launch": alg_bytes,
-                         "kernel": {"panel": "k_panel", "panel_pb": "k_panel_pb", "panel_w": "k_panel_w", "panel_q": "k_panel_q"}.get(
-                             op.compile(theta.detach()).path,
-                             "k_matvec_q2_fx" if args.dtype == "f64" else "k_matvec_q2_f32x") + " + k_term_grads",
+                         "kernel": KERNELS.get(op.compile(theta.detach()).kernel(x.dtype),
+                                               "k_matvec_q2_fx" if args.dtype == "f64" else "k_matvec_q2_f32x") +
+                         " + k_grad_panel",  # the workload's partition (12 + 12 sites, one column)
                          "main_kernels_ms_per_step": kern_ms / args.steps},
             "clocks": clk.summary(),
             "gpu_launches": kernels,
@@ -636,11 +640,9 @@ def main():
             dist.barrier()
         torch.cuda.synchronize()
 
-    path = t.path if args.nrhs == 1 else "general"
     general = (("k_matvec_q2_fx" if args.dtype == "f64" else "k_matvec_q2_f32x") if w.Q == 2 else
                ("k_matvec_qg_fx" if args.dtype == "f64" else "k_matvec_qg_f32x"))
-    kernel_name = {"panel": "k_panel", "panel_pb": "k_panel_pb", "panel_w": "k_panel_w", "panel_q": "k_panel_q",
-                   "cluster": "k_matvec_cl"}.get(path, general)
+    kernel_name = KERNELS.get(t.kernel(tdtype, args.nrhs), general)
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     with ClockSampler(local) as clk:
         barrier()

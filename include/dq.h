@@ -160,7 +160,7 @@ int dq_check_device(const dq_sector* s, void* stream);
  * (dq_free_terms). Synchronous. */
 int dq_make_terms(const dq_sector* s, const dq_term* terms, int n_terms, dq_terms** out);
 
-/* Which product kernel dq_matvec uses for these terms with one right-hand side: *path = 1 for the
+/* The form of the product for these terms with one right-hand side: *path = 1 for the
  * panel kernel (Q = 2, uniform single-site fields, at most two distinct hop amplitudes and four
  * distinct Sz Sz coefficients, dyadic coefficients; either two subsystems with P_1 of at most 15
  * sites and P_0 of at most 16, or three or more subsystems whose last one has fewer than 8 or more
@@ -182,8 +182,14 @@ int dq_make_terms(const dq_sector* s, const dq_term* terms, int n_terms, dq_term
  * it gives the general kernel's y). The values 0, 1 and 4 name the form that fits the sector's own
  * partition; sectors of at least 2^19 rows whose own panels are of fewer than 15 sites run the panel
  * kernel on the lowest 15 sites (L - 9 below 24 sites) instead where the operator fits it, with the
- * same y. */
+ * same y (dq_matvec_kernel tells). */
 int dq_terms_path(const dq_terms* t, int* path);
+
+/* The kernel that dq_matvec launches for these terms, vectors of `dtype` and `nrhs` right-hand
+ * sides: *kernel = 0 to 5 as the values of dq_terms_path, or 6 for the panel kernel on the lowest
+ * sites of the lattice in place of the sector's own partition. Errors: DQ_EINVAL for NULL, a bad
+ * dtype or nrhs outside [1, 64]. */
+int dq_matvec_kernel(const dq_terms* t, int dtype, int nrhs, int* kernel);
 
 /* Compile terms in the cluster-merged form of App. C instead: the terms are grouped into clusters
  * of at most `cluster_sites` sites (clusters may overlap; each term goes to the first cluster that

@@ -29,7 +29,7 @@ EXPORTED = (
     "dq_last_error", "dq_make_sector", "dq_free_sector", "dq_sector_dim", "dq_sector_partition",
     "dq_state_at", "dq_index_of", "dq_next_state", "dq_state_at_batch", "dq_index_of_batch",
     "dq_state_at2", "dq_index_of2", "dq_next_state2", "dq_state_at_batch2", "dq_index_of_batch2",
-    "dq_check_device", "dq_make_terms", "dq_terms_path", "dq_free_terms", "dq_matvec", "dq_matvec_noalloc",
+    "dq_check_device", "dq_make_terms", "dq_terms_path", "dq_matvec_kernel", "dq_free_terms", "dq_matvec", "dq_matvec_noalloc",
     "dq_lanczos", "dq_make_cluster_terms", "dq_cluster_info", "dq_batch_make", "dq_batch_matvec", "dq_batch_tune", "dq_batch_shape", "dq_batch_free", "dq_term_grads",
     "dq_timing_enable", "dq_timing_read",
 )
@@ -73,6 +73,7 @@ def _load() -> ctypes.CDLL:
         "dq_make_cluster_terms": (i32, [vp, P(_Term), i32, i32, P(vp)]),
         "dq_cluster_info": (i32, [vp, P(i32), P(i32), P(i32)]),
         "dq_terms_path": (i32, [vp, P(i32)]),
+        "dq_matvec_kernel": (i32, [vp, i32, i32, P(i32)]),
         "dq_matvec": (i32, [vp, vp, vp, vp, i32, i32, vp]),
         "dq_matvec_noalloc": (i32, [vp, vp, vp, vp, i32, vp]),
         "dq_batch_make": (i32, [i32, P(vp), P(vp), i32, i32, P(vp)]),
@@ -239,6 +240,9 @@ def next_state(sector: Sector, state: int) -> int:
     return sector.next_state(state)
 
 
+_KERNELS = ("general", "panel", "cluster", "panel_pb", "panel_w", "panel_q", "panel_split")
+
+
 class Terms:
     """Operator terms compiled for one sector; ``terms`` is a list of (kind, i, j, coef). With
     ``cluster_sites`` the cluster-merged form of App. C (dq_make_cluster_terms)."""
@@ -271,11 +275,19 @@ class Terms:
 
     @property
     def path(self) -> str:
-        """'panel', 'panel_pb', 'panel_w', 'panel_q', 'general' or 'cluster': the product kernel used
-        for one right-hand side."""
+        """'panel', 'panel_pb', 'panel_w', 'panel_q', 'general' or 'cluster': the form of the product
+        that fits the sector's own partition, for one right-hand side (``kernel`` names what runs)."""
         v = ctypes.c_int()
         _check(_lib.dq_terms_path(self._h, ctypes.byref(v)))
-        return {1: "panel", 2: "cluster", 3: "panel_pb", 4: "panel_w", 5: "panel_q"}.get(v.value, "general")
+        return _KERNELS[v.value]
+
+    def kernel(self, dtype, nrhs: int = 1) -> str:
+        """The kernel that ``matvec`` launches for vectors of this dtype and number of right-hand sides:
+        the names of ``path``, or 'panel_split' for the panel kernel on the lattice's lowest sites in
+        place of the sector's own partition."""
+        v = ctypes.c_int()
+        _check(_lib.dq_matvec_kernel(self._h, _code_of(dtype), int(nrhs), ctypes.byref(v)))
+        return _KERNELS[v.value]
 
     def __del__(self):
         h = getattr(self, "_h", None)
@@ -292,14 +304,18 @@ def make_cluster_terms(sector: Sector, terms, cluster_sites: int) -> Terms:
     return Terms(sector, terms, cluster_sites)
 
 
-def _dtype_code(t) -> int:
+def _code_of(dtype) -> int:
     import torch
 
-    if t.dtype == torch.float64:
+    if dtype == torch.float64:
         return DQ_F64
-    if t.dtype == torch.float32:
+    if dtype == torch.float32:
         return DQ_F32
     raise TypeError("vectors must be float64 or float32")
+
+
+def _dtype_code(t) -> int:
+    return _code_of(t.dtype)
 
 
 def _check_vec(sector: Sector, t, name: str):

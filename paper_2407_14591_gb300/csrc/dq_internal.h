@@ -359,6 +359,9 @@ int launch_rank_long(const DevSector& S, bool inverse, const uint64_t* in, uint6
 int launch_state_at_batch(const DevSector& S, const uint64_t* d_index, uint64_t* d_state, uint64_t n, void* stream);
 int launch_index_of_batch(const DevSector& S, const uint64_t* d_state, uint64_t* d_index, uint64_t n, void* stream);
 int launch_matvec(const dq_sector* s, const dq_terms* t, const void* x, void* y, int dtype, int nrhs, void* stream);
+// Product kernels, numbered as in dq_matvec_kernel; the one that a product runs (dq_terms.cpp).
+enum MatvecKernel { kMvGeneral = 0, kMvPanel = 1, kMvCluster = 2, kMvPanelPB = 3, kMvPanelW = 4, kMvPanelQ = 5, kMvSplit = 6 };
+MatvecKernel matvec_kernel(const dq_terms* t, int dtype, int nrhs);
 // the same batches for states stored as two uint64 words (low word first)
 int launch_state_at_batch_w(const DevSector& S, const uint64_t* d_index, uint64_t* d_state, uint64_t n, void* stream);
 int launch_index_of_batch_w(const DevSector& S, const uint64_t* d_state, uint64_t* d_index, uint64_t n, void* stream);

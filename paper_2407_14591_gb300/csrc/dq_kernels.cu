@@ -443,20 +443,18 @@ static int launch_matvec_f32x(const dq_sector* s, dq_terms* t, const float* x, f
 
 int launch_matvec(const dq_sector* s, const dq_terms* t, const void* x, void* y, int dtype, int nrhs, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    if (t->cluster) return launch_cluster_matvec(s, const_cast<dq_terms*>(t), x, y, dtype, nrhs, stream);
-    if ((t->panel_ok || t->split) && nrhs == 1) return launch_panel_matvec(s, const_cast<dq_terms*>(t), x, y, dtype, stream);
-    if (t->pw_ok && nrhs == 1) return launch_panel_w(s, const_cast<dq_terms*>(t), x, y, dtype, stream);
-    if (t->pq_ok && nrhs == 1) return launch_panel_q(s, const_cast<dq_terms*>(t), x, y, dtype, stream);
-    // Per-bond panels, column by column. The general kernel shares the rank of a hop among the columns, so
-    // it wins with many of them; it loses with few on long vectors (measured, us, general against panels:
-    // 23 sites 217 / 139 with two FP64 columns, 277 / 207 with three; 26 sites 1763 / 779, 2336 / 1168 and
-    // 4365 / 3120 with eight; FP32 1381 / 569 and 1506 / 841, but 2283 / 2255 with eight; 21 sites, D =
-    // 203,490: 45 / 55 with two).
-    if (t->pb_ok && (nrhs == 1 || (nrhs <= 3 && s->D >= (1u << 19)) ||
-                     (nrhs <= 8 && dtype == DQ_F64 && s->D >= (1u << 21))))
-        return launch_panel_pb(s, const_cast<dq_terms*>(t), x, y, dtype, nrhs, stream);
-    if (dtype == DQ_F64) return launch_matvec_fx(s, const_cast<dq_terms*>(t), (const double*)x, (double*)y, nrhs, st);
-    return launch_matvec_f32x(s, const_cast<dq_terms*>(t), (const float*)x, (float*)y, nrhs, st);
+    dq_terms* tw = const_cast<dq_terms*>(t);
+    switch (matvec_kernel(t, dtype, nrhs)) {
+        case kMvCluster: return launch_cluster_matvec(s, tw, x, y, dtype, nrhs, stream);
+        case kMvPanel:
+        case kMvSplit: return launch_panel_matvec(s, tw, x, y, dtype, stream);
+        case kMvPanelW: return launch_panel_w(s, tw, x, y, dtype, stream);
+        case kMvPanelQ: return launch_panel_q(s, tw, x, y, dtype, stream);
+        case kMvPanelPB: return launch_panel_pb(s, tw, x, y, dtype, nrhs, stream);
+        default: break;
+    }
+    if (dtype == DQ_F64) return launch_matvec_fx(s, tw, (const double*)x, (double*)y, nrhs, st);
+    return launch_matvec_f32x(s, tw, (const float*)x, (float*)y, nrhs, st);
 }
 
 }  // namespace dq

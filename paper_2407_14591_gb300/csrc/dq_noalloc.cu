@@ -72,9 +72,10 @@ extern "C" int dq_matvec_noalloc(const dq_sector* s, const dq_terms* t, const vo
     void* ws = nullptr;
     int rc = noalloc_scratch(&ws);
     if (rc) return rc;
-    int e = t->panel_ok || t->split ? launch_panel_matvec_ws(s, t, x, y, dtype, ws, stream)
-            : t->pw_ok ? launch_panel_w_ws(s, t, x, y, dtype, ws, stream)
-                        : launch_panel_q_ws(s, t, x, y, dtype, ws, stream);
+    const MatvecKernel k = matvec_kernel(t, dtype, 1);
+    int e = k == kMvPanelW   ? launch_panel_w_ws(s, t, x, y, dtype, ws, stream)
+            : k == kMvPanelQ ? launch_panel_q_ws(s, t, x, y, dtype, ws, stream)
+                             : launch_panel_matvec_ws(s, t, x, y, dtype, ws, stream);
     if (e) return set_error(DQ_ECUDA, "matvec_noalloc launch: %s", cudaGetErrorString((cudaError_t)e));
     return DQ_OK;
 }
