@@ -181,8 +181,8 @@ int dq_make_terms(const dq_sector* s, const dq_term* terms, int n_terms, dq_term
  * coefficient per hop bond and any site function (the per-term form's integer coefficients, so
  * it gives the general kernel's y). The values 0, 1 and 4 name the form that fits the sector's own
  * partition; sectors of at least 2^19 rows whose own panels are of fewer than 15 sites run the panel
- * kernel on the lowest 15 sites (L - 9 below 24 sites) instead where the operator fits it, with the
- * same y (dq_matvec_kernel tells). */
+ * kernel on the lowest 15 sites (L - 9 below 24 sites) instead where the operator fits it and, unless
+ * the own form is 1, its panels hold 320 rows on average, with the same y (dq_matvec_kernel tells). */
 int dq_terms_path(const dq_terms* t, int* path);
 
 /* The kernel that dq_matvec launches for these terms, vectors of `dtype` and `nrhs` right-hand

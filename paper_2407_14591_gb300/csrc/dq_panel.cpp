@@ -140,9 +140,24 @@ static int split_sites(const dq_sector* s) { return std::min(15, s->L - 9); }
 // (13) 2626 -> 1447, 2379 -> 1169; 7 x 4 lattice (14) 3519 -> 2946, 3048 -> 2354; chain of 24 sites (12)
 // 103 -> 90, 99 -> 80; chain of 22 sites, 0.7 M rows (11 against 13) 54 -> 47, 49 -> 43. Of equal length
 // the own form is faster (7 x 4 with P_1 of 14 sites in the split order: 3569 and 3104).
-static bool use_split_order(const dq_sector* s, int own_sites) {
+//
+// A block's frame around a panel is the same for a short one, so where the alternative is not this kernel
+// with fewer sites (own_panel) but one warp per panel or the general kernel, the panels have to hold 320
+// rows on average. J1-J2 chains with three subsystems, FP64, warp panels against split order: 49 rows (31
+// sites, N = 6) 294 / 784 us, 204 rows (28, 7) 313 / 378, 257 (30, 8) 1057 / 1442, 269 (27, 7) 228 / 244,
+// 362 (26, 7) 210 / 161, 438 (28, 8) 611 / 499, 1068 (25, 8) 228 / 134; the 9 x 3 lattice (27, 7), general
+// kernel against split order, 348 / 471.
+constexpr uint64_t kSplitMinRows = 320;
+static bool use_split_order(const dq_sector* s, int own_sites, bool own_panel) {
     const int L1 = split_sites(s);
-    return s->D >= kSplitMinDim && s->D < (1ull << 48) && L1 > 10 && L1 > own_sites && s->L - L1 <= 16;
+    if (s->D < kSplitMinDim || s->D >= (1ull << 48) || L1 <= 10 || L1 <= own_sites || s->L - L1 > 16) return false;
+    if (own_panel) return true;
+    uint64_t panels = 0, c = 1;  // c = C(L - L1, n0)
+    for (int n0 = 0; n0 <= s->L - L1; ++n0) {
+        if (s->N - n0 >= 0 && s->N - n0 <= L1) panels += c;
+        c = c * (s->L - L1 - n0) / (n0 + 1);
+    }
+    return s->D >= kSplitMinRows * panels;
 }
 
 // Bits of the lowest whole subsystems inside a suffix of L1 bits (L1 itself when the suffix lies
@@ -578,9 +593,9 @@ int build_panel_plan(const dq_sector* s, double C, bool uniform_lin,
     bool own = false;
     if (int rc = build_form(s, C, pairs, t, false, true, &own)) return rc;
     const int ns = s->n_sub, last = s->Lk[ns - 1];
-    const bool tail = ns >= 3 && (last < 8 || last > 10);
+    const bool warp = last >= 8 && last <= 10, tail = ns >= 3 && !warp;
     const int own_sites = !own ? 0 : tail ? s->Lk[ns - 2] + last : last;
-    if (use_split_order(s, own_sites) && (own || ns >= 3)) {
+    if ((own || ns >= 3) && use_split_order(s, own_sites, own && !warp)) {
         if (int rc = build_form(s, C, pairs, t, true, true, &fits)) return rc;
         if (fits) {
             if (int rc = build_form(s, C, pairs, t, true, false, &fits)) return rc;

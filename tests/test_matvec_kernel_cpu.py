@@ -53,3 +53,23 @@ def test_cluster_terms_and_bad_arguments():
     assert b.lib().dq_matvec_kernel(None, b.DQ_F64, 1, ctypes.byref(ctypes.c_int())) == b.DQ_EINVAL
     assert b.lib().dq_matvec_kernel(t.handle, 7, 1, ctypes.byref(ctypes.c_int())) == b.DQ_EINVAL
     assert b.lib().dq_matvec_kernel(t.handle, b.DQ_F64, 1, None) == b.DQ_EINVAL
+
+
+@pytest.mark.parametrize("L,N,n_sub,terms,kernel", [
+    # the split order's panels are mostly short: 49, 60, 204, 257 and 269 rows on average
+    (31, 6, 3, chain(31), "panel_w"),
+    (30, 6, 3, chain(30), "panel_w"),
+    (28, 7, 3, chain(28), "panel_w"),
+    (30, 8, 3, chain(30), "panel_w"),
+    (27, 7, 3, lattice(9, 3), "general"),
+    # 362 and 438 rows
+    (26, 7, 3, chain(26), "panel_split"),
+    (28, 8, 3, chain(28), "panel_split"),
+    # against a tail or two subsystems of fewer sites it wins at any length: 49 and 158 rows
+    (31, 6, 5, chain(31), "panel_split"),
+    (29, 7, 2, chain(29), "panel_split"),
+])
+def test_split_order_only_where_its_panels_are_long(L, N, n_sub, terms, kernel):
+    s = b.make_sector(L, 2, N, n_sub)
+    assert s.dim >= 1 << 19
+    assert b.make_terms(s, terms).kernel(torch.float64) == kernel
