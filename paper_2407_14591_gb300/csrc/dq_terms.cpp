@@ -449,12 +449,20 @@ MatvecKernel matvec_kernel(const dq_terms* t, int dtype, int nrhs) {
         if (t->pq_ok) return kMvPanelQ;
     }
     // Per-bond panels, column by column. The general kernel shares the rank of a hop among the columns, so
-    // it wins with many of them; it loses with few on long vectors (measured, us, general against panels:
-    // 23 sites 217 / 139 with two FP64 columns, 277 / 207 with three; 26 sites 1763 / 779, 2336 / 1168 and
-    // 4365 / 3120 with eight; FP32 1381 / 569 and 1506 / 841, but 2283 / 2255 with eight; 21 sites, D =
-    // 203,490: 45 / 55 with two).
+    // it wins with many of them and, as a block's frame around a panel is the same for a short one, at low
+    // filling. Measured, us, general against panels, by rows a panel (D / panels):
+    //   two columns, FP64: 113 rows (26 sites, N = 7) 112 / 166, 172 (27, 8) 351 / 397, 203 (23, 9) 146 / 132,
+    //     280 (23, 10) 196 / 144, 660 (24, 12) 434 / 251; 21 sites, D = 203,490: 45 / 55;
+    //   three: 194 (24, 8) 148 / 175, 220 (26, 8) 310 / 356, 262 (25, 9) 409 / 389, 660 558 / 365; FP32, whose
+    //     general kernel has cheaper columns: 262 276 / 316, 314 (27, 9) 627 / 694, 330 (23, 11) 198 / 186;
+    //   FP64, four: 314 1053 / 1119, 404 (25, 10) 753 / 662; eight: 404 1285 / 1324, 530 (27, 10) 3411 / 3288,
+    //     660 1024 / 945, 1270 (26, 13) 4365 / 3120; FP32, eight: 1270 2283 / 2255.
     const uint64_t D = t->sector->D;
-    if (t->pb_ok && (nrhs == 1 || (nrhs <= 3 && D >= (1u << 19)) || (nrhs <= 8 && dtype == DQ_F64 && D >= (1u << 21))))
+    const bool f64 = dtype == DQ_F64;
+    auto rows = [&](uint64_t least) { return D >= least * t->pbp.npanels; };
+    if (t->pb_ok && (nrhs == 1 || (nrhs == 2 && D >= (1u << 19) && rows(200)) ||
+                     (nrhs == 3 && D >= (1u << 19) && rows(f64 ? 256 : 330)) ||
+                     (nrhs <= 8 && nrhs > 3 && f64 && D >= (1u << 21) && rows(nrhs == 4 ? 350 : 500))))
         return kMvPanelPB;
     return kMvGeneral;
 }

@@ -73,3 +73,23 @@ def test_split_order_only_where_its_panels_are_long(L, N, n_sub, terms, kernel):
     s = b.make_sector(L, 2, N, n_sub)
     assert s.dim >= 1 << 19
     assert b.make_terms(s, terms).kernel(torch.float64) == kernel
+
+
+@pytest.mark.parametrize("L,N,f64,f32", [
+    # columns up to which a product of a disordered chain takes the per-bond panels
+    (26, 7, 1, 1),    # 113 rows a panel on average
+    (27, 8, 1, 1),    # 172
+    (23, 9, 2, 2),    # 203
+    (25, 9, 3, 2),    # 262
+    (23, 10, 3, 2),   # 280
+    (27, 9, 3, 2),    # 314, 4.7 M rows
+    (23, 11, 3, 3),   # 330
+    (25, 10, 4, 3),   # 404, 3.3 M rows
+    (24, 10, 3, 3),   # 480, but 2.0 M rows
+    (24, 12, 8, 3),   # 660
+])
+def test_columns_of_the_per_bond_panels(L, N, f64, f32):
+    t = b.make_terms(b.make_sector(L, 2, N, 2), xxz(L))
+    for dtype, most in ((torch.float64, f64), (torch.float32, f32)):
+        got = [c for c in range(1, 65) if t.kernel(dtype, c) == "panel_pb"]
+        assert got == list(range(1, most + 1)), dtype
