@@ -445,8 +445,26 @@ __global__ void k_grad_fixed(const T* __restrict__ x, const T* __restrict__ dy, 
 
 // ------------------------------------------------------------------ host --------------------
 
-// The plan for a term list; false when it does not fit (too many pairs of one place, or the sector).
-static bool grad_plan(const dq_sector* s, const dq_term* terms, int n_terms, GradPlan& P, std::vector<GradOut>& outs) {
+// Where the pass over panels pays. It works on the columns one after the other, the general kernels rank a
+// hop once for all columns; it shares a panel's loads among all terms; and its frame around a panel is the
+// same for a short one. With one column it is always the faster. Measured, us, general against panels, by
+// rows a panel:
+//   little work, bound by launches: 20 sites, N = 6 (46 rows), four columns 297 / 216; N = 10 (180), eight
+//     413 / 345, sixteen and eight terms 251 / 245; 24 sites, N = 6 (54), two 416 / 299, three and 24 terms 194 / 235;
+//   few terms: 24 sites, N = 12 (660 rows), eight terms and four columns 432 / 387, eight columns 640 / 680;
+//     N = 9 (325) two 239 / 187, four 283 / 304; 26 sites, N = 6 (56) two 168 / 154 but 78 terms 453 / 602;
+//   many terms: 24 sites, N = 12, 72 terms, eight columns 4164 / 1648, 24 terms and sixteen 3588 / 2490; N = 9,
+//     72 terms and sixteen 3762 / 2602, eight terms 794 / 1082; 26 sites, N = 9 (400), 78 terms and sixteen 8999 /
+//     9201; 22 sites, N = 11 (344), 66 terms and 32 3551 / 2967, eight terms 881 / 1525.
+static bool grad_pays(uint64_t D, uint32_t npanels, int n_terms, int cols) {
+    const uint64_t rows = D / npanels, items = (uint64_t)npanels * cols;
+    return cols == 1 || items <= (rows >= 150 ? 8192 : 5120) || (cols <= 4 && rows >= 160 * (uint64_t)cols) ||
+           (cols <= 16 && rows >= 300 && (uint64_t)n_terms * rows >= 9600);
+}
+
+// The plan for a term list; false when it does not fit (too many pairs of one place, or the sector) or
+// would not pay.
+static bool grad_plan(const dq_sector* s, const dq_term* terms, int n_terms, int cols, GradPlan& P, std::vector<GradOut>& outs) {
     if (s->Q != 2 || s->n_sub != 2 || s->wide) return false;
     const int L = s->L, L0 = s->Lk[0], L1 = s->Lk[1], N = s->N;
     if (L1 < 1 || L1 > 13 || L0 > 16) return false;
@@ -459,6 +477,7 @@ static bool grad_plan(const dq_sector* s, const dq_term* terms, int n_terms, Gra
     const int a = std::max(0, N - L1), b = std::min(L0, N);  // particle numbers of P_0
     P.s0 = s->dev.unrank_tab[s->dev.tab[0]] + s0s[a];
     P.npanels = s0s[b + 1] - s0s[a];
+    if (!grad_pays(s->D, P.npanels, n_terms, cols)) return false;
     P.c0 = s->dev.c0_tab;
     P.rank1 = s->dev.rank_tab[s->dev.tab[1]];
     P.states = s->dev.unrank_tab[s->dev.tab[1]];
@@ -552,7 +571,7 @@ int launch_grad_panel(const dq_sector* s, const dq_term* terms, int n_terms, con
                       int cols, double* d_grads, cudaStream_t st, bool* taken) {
     GradPlan P;
     std::vector<GradOut> outs;
-    *taken = grad_plan(s, terms, n_terms, P, outs);
+    *taken = grad_plan(s, terms, n_terms, cols, P, outs);
     if (!*taken) return 0;
     const GradSmem L(P);
     const int sms = sm_count_cached();
