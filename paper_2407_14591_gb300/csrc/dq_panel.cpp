@@ -476,21 +476,40 @@ static int build_form(const dq_sector* s, double C,
     auto start_of = [&](uint32_t p) -> uint64_t { return tail_start.empty() ? s->h.c0_tab[p] : tail_start[p]; };
     P.npanels = (uint32_t)ps0.size();
     P.cmax = cmax;
-    // per-panel diagonal (see PanelRowDiag) and the P_1 Sz Sz sums of the patterns
+    // per-panel diagonal (see PanelRowDiag) and the P_1 Sz Sz sums of the patterns. A panel's sums are built up
+    // over the set bits of s0, lowest first: setting bit a changes [s_a != s_j] of its bonds inside P_0 by
+    // 1 - 2 s_j, and turns its bonds across the cut from s_b to 1 - s_b.
     std::vector<PanelRowDiag> pdiag(ps0.size());
+    uint32_t nb[32][kPanelMaxK] = {};  // P_0 bits with a bond of class k to bit a
+    std::vector<std::vector<std::pair<int, long long>>> cut(32);
+    PanelRowDiag none;  // s0 = 0
+    std::memset(&none, 0, sizeof none);
+    none.pd = P.MC;
+    for (int k = 0; k < P.nK; ++k) {
+        for (int l = (k ? P.p0z_end[k - 1] : 0); l < P.p0z_end[k]; ++l) {
+            const uint32_t lo = P.p0z_mask[l] & (~P.p0z_mask[l] + 1u), hi = P.p0z_mask[l] ^ lo;
+            nb[__builtin_ctz(lo)][k] |= hi;
+            nb[__builtin_ctz(hi)][k] |= lo;
+        }
+        for (int l = (k ? P.xz_end[k - 1] : 0); l < P.xz_end[k]; ++l) {
+            const int bit = __builtin_ctz(P.xz_bbit[l]);
+            none.w[bit] += P.MK[k];
+            cut[__builtin_ctz(P.xz_abit[l])].push_back({bit, P.MK[k]});
+        }
+    }
     for (size_t q = 0; q < ps0.size(); ++q) {
-        const uint32_t s0 = ps0[q];
         PanelRowDiag& g = pdiag[q];
-        std::memset(&g, 0, sizeof g);
-        g.pd = P.MC;
-        for (int k = 0; k < P.nK; ++k) {
-            for (int l = (k ? P.p0z_end[k - 1] : 0); l < P.p0z_end[k]; ++l)
-                if (__builtin_popcount(s0 & P.p0z_mask[l]) == 1) g.pd += P.MK[k];
-            for (int l = (k ? P.xz_end[k - 1] : 0); l < P.xz_end[k]; ++l) {
-                const bool sa = (s0 & P.xz_abit[l]) != 0;
-                if (sa) g.pd += P.MK[k];
-                g.w[__builtin_ctz(P.xz_bbit[l])] += sa ? -P.MK[k] : P.MK[k];
+        g = none;
+        uint32_t below = 0;
+        for (uint32_t m = ps0[q]; m; m &= m - 1) {
+            const int at = __builtin_ctz(m);
+            for (int k = 0; k < P.nK; ++k)
+                g.pd += P.MK[k] * (__builtin_popcount(nb[at][k]) - 2 * __builtin_popcount(nb[at][k] & below));
+            for (auto& e : cut[at]) {
+                g.pd += e.second;
+                g.w[e.first] -= 2 * e.second;
             }
+            below |= 1u << at;
         }
     }
     std::vector<long long> d1(t1states.size(), 0);

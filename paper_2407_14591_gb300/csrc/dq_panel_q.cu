@@ -107,6 +107,7 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
         std::vector<std::vector<uint32_t>> lists(C1);
         size_t mx = 0;
         for (uint32_t c = 0; c < C1; ++c) {
+            lists[c].reserve(d1.size());
             const uint32_t s1 = ut[b0 + c];
             long long dg = 0;
             for (int q = 0; q < nsite; ++q)
@@ -168,9 +169,11 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
     std::vector<uint32_t> loff(pl.size() + 1, 0), lhdr(pl.size(), 0);
     std::vector<uint64_t> lst;
     lst.reserve(pl.size() * (d0.size() + dx.size()));
+    std::vector<int> num(pl.size(), 0);  // particles of P_0
     auto digit0 = [&](uint32_t s0, int sh) { return (int)((s0 >> sh) & dm); };
     for (size_t i = 0; i < pl.size(); ++i) {
         const uint32_t s0 = pl[i].second;
+        for (int k = 0; k < L0; ++k) num[i] += digit0(s0, nb * k);
         ps0[i] = s0;
         pst[i] = pl[i].first.second;
         long long dg = MC;
@@ -214,34 +217,27 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
     // single, cut into pieces, full pieces first. The pieces are as long as leaves every resident warp four
     // units, and the panels are paired while it leaves one: on smaller sectors a unit's length is the
     // product's time (44,473 rows: pieces of 4, 2 chunks of pairs 36, 28 us; 8451 rows: pairs 24, single 20 us).
-    auto n_of = [&](uint32_t s0) {
-        int n = 0;
-        for (int k = 0; k < L0; ++k) n += digit0(s0, nb * k);
+    std::vector<unsigned char> pairs(pl.size());  // panel i starts a pair
+    for (size_t i = 0; i + 1 < pl.size(); i += 1 + pairs[i]) pairs[i] = num[i] == num[i + 1];
+    auto chunks_of = [&](size_t i) { return (~pl[i].first.first + 31) / 32; };
+    auto count = [&](uint32_t chunks) {  // units of pairs
+        size_t n = 0;
+        for (size_t i = 0; i < pl.size(); i += 1 + pairs[i]) n += (chunks_of(i) + chunks - 1) / chunks;
         return n;
-    };
-    std::vector<uint64_t> units;
-    auto cut = [&](bool pair, uint32_t chunks) {
-        std::vector<std::vector<uint64_t>> unit(chunks + 1);
-        for (size_t i = 0; i < pl.size();) {
-            const bool two = pair && i + 1 < pl.size() && n_of(ps0[i]) == n_of(ps0[i + 1]);
-            const uint32_t ch = (~pl[i].first.first + 31) / 32;
-            for (uint32_t c = 0; c < ch; c += chunks) {
-                const uint32_t len = std::min(chunks, ch - c);
-                unit[len].push_back((uint64_t)i | ((uint64_t)c << 32) | ((uint64_t)len << 48) | ((uint64_t)two << 63));
-            }
-            i += two ? 2 : 1;
-        }
-        units.clear();
-        for (uint32_t len = chunks; len > 0; --len) units.insert(units.end(), unit[len].begin(), unit[len].end());
     };
     const size_t warps = (size_t)sm_count_cached() * 2 * kPQW;
     uint32_t chunks = kPQChunks;
-    P.pairs = 1;
-    for (cut(true, chunks); chunks > 1 && units.size() < 4 * warps; cut(true, chunks)) chunks /= 2;
-    if (units.size() < warps) {
-        P.pairs = 0;
-        cut(false, chunks);
-    }
+    while (chunks > 1 && count(chunks) < 4 * warps) chunks /= 2;
+    P.pairs = count(chunks) >= warps;
+    if (!P.pairs) std::fill(pairs.begin(), pairs.end(), 0);
+    std::vector<std::vector<uint64_t>> unit(chunks + 1);
+    for (size_t i = 0; i < pl.size(); i += 1 + pairs[i])
+        for (uint32_t c = 0, ch = chunks_of(i); c < ch; c += chunks) {
+            const uint32_t len = std::min(chunks, ch - c);
+            unit[len].push_back((uint64_t)i | ((uint64_t)c << 32) | ((uint64_t)len << 48) | ((uint64_t)pairs[i] << 63));
+        }
+    std::vector<uint64_t> units;
+    for (uint32_t len = chunks; len > 0; --len) units.insert(units.end(), unit[len].begin(), unit[len].end());
     P.nunits = (uint32_t)units.size();
     int rc;
     void* p;
@@ -260,14 +256,20 @@ int build_panel_q(const dq_sector* s, const std::vector<int>& site_sh, const std
     if ((rc = up(pst.data(), pst.size() * 8, (const void**)&P.panel_start))) return rc;
     if ((rc = up(mh.data(), mh.size() * 8, (const void**)&P.Mhop))) return rc;
     if ((rc = up(rdiag.data(), rdiag.size() * 8, (const void**)&P.rdiag))) return rc;
+    // an upload is an allocation and a copy, most of the plan's time on small sectors: the units stand behind
+    // the source lists, the slot counts behind the P_1 lists
+    const size_t nlst = lst.size(), nell = p1ell.size();
+    lst.insert(lst.end(), units.begin(), units.end());
+    p1ell.resize(nell + (p1cnt.size() + 3) / 4);
+    if (!p1cnt.empty()) std::memcpy(p1ell.data() + nell, p1cnt.data(), p1cnt.size());
     if ((rc = up(p1ell.data(), p1ell.size() * 4, (const void**)&P.p1ell))) return rc;
+    P.p1cnt = reinterpret_cast<const unsigned char*>(P.p1ell + nell);
     if ((rc = up(cutt.data(), cutt.size() * 4, (const void**)&P.cutt))) return rc;
-    if ((rc = up(units.data(), units.size() * 8, (const void**)&P.unit))) return rc;
-    if ((rc = up(p1cnt.data(), p1cnt.size(), (const void**)&P.p1cnt))) return rc;
     if ((rc = up(pdiag.data(), pdiag.size() * 8, (const void**)&P.pdiag))) return rc;
     if ((rc = up(loff.data(), loff.size() * 4, (const void**)&P.list_off))) return rc;
     if ((rc = up(lhdr.data(), lhdr.size() * 4, (const void**)&P.list_hdr))) return rc;
     if ((rc = up(lst.data(), lst.size() * 8, (const void**)&P.list))) return rc;
+    P.unit = P.list + nlst;
     t->pq_ok = P.npanels > 0;
     return DQ_OK;
 }
