@@ -173,7 +173,7 @@ struct PanelPlan {
     const uint64_t* list;
     const PanelRowDiag* diag;   // per panel
     const long long* d1;        // P_1 Sz Sz of every P_1 pattern, in the order of t1states
-    // three or more subsystems (the warp-panel kernel): prefix bits of the Sz Sz bonds across the
+    // the warp-panel kernel: prefix bits of the Sz Sz bonds across the
     // cut, per class and per position b of P_1 (the per-panel counters are built on the device)
     uint32_t xzA[kPanelMaxK][32];
     // split order (dq_panel.cpp): canonical index of a row = piece[panel * npiece + (rowy >> 16)] +
@@ -281,11 +281,11 @@ struct PanelQ {
                                   // row part of the Mhop entry << 16 | (the hop is not allowed) << 31
     uint32_t cutbase[kPQMaxN + 1];
     const long long* pdiag;       // per panel: the constant plus the P_0 site functions
-    // per-panel sources: P_0 partners (start | Mhop entry << 40), then cut partners
-    // (start | cut direction << 40 | panel part of the Mhop entry << 48)
     // work of a warp: panel | first 32-row chunk << 32 | chunks << 48 | the next panel too << 63
     const uint64_t* unit;
     uint32_t nunits, pairs;       // pairs: units are of two panels
+    // per-panel sources: P_0 partners (start | Mhop entry << 40), then cut partners
+    // (start | cut direction << 40 | panel part of the Mhop entry << 48)
     const uint32_t* list_off;
     const uint32_t* list_hdr;     // bits 0-7: P_0 entries, 8-15: cut entries
     const uint64_t* list;
@@ -324,9 +324,9 @@ struct dq_terms {
     std::vector<void*> dev_allocs;
     int max_hops;  // upper bound on off-diagonal elements per row
     bool panel_ok = false;     // the panel product applies (see PanelPlan)
-    bool split = false;        // the panel kernel runs on the split order (three or more subsystems)
+    bool split = false;        // the panel kernel runs on the split order (dq_panel.cpp)
     bool pb_ok = false;        // the per-bond panel product applies (PanelPB)
-    bool pw_ok = false;        // the warp-panel product applies (three or more subsystems, PanelPlan)
+    bool pw_ok = false;        // the warp-panel product applies (PanelPlan)
     bool pq_ok = false;        // the boson panel product applies (Q > 2, PanelQ)
     dq::PanelQ pqp;
     dq::PanelPB pbp;

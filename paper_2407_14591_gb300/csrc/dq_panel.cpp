@@ -28,7 +28,8 @@
 // the tail's particle number only; the host tabulates it (tail pattern -> local index) from the
 // sector's own rank and checks every panel's first and last row.
 //
-// Large sectors whose own panels are of fewer than 15 sites take neither: the panel kernel works on x in
+// Large sectors whose own panels are of fewer than 15 sites take neither (use_split_order below has the
+// rule): the panel kernel works on x in
 // the order of a split into TWO subsystems of its own (the "split order": P_0 = the upper L - L_1 sites,
 // P_1 the lower L_1 <= 15), whatever the sector's partition is. The prepass that makes the fixed-point
 // copy of x gathers it into that order and the kernel's stores go back through the same map. A panel of

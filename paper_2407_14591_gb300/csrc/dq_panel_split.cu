@@ -1,4 +1,4 @@
-// The panel product on the split order (three or more subsystems; see dq_panel.cpp): the table of
+// The panel product on the split order (any number of subsystems; see dq_panel.cpp): the table of
 // canonical pieces and the kernels of dq_panel.cuh with the mapped stores.
 #include "dq_panel.cuh"
 

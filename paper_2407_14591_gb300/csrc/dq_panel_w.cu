@@ -1,4 +1,5 @@
-// Warp-panel product y = H x for Q = 2 and three or more subsystems (plan in dq_panel.cpp).
+// Warp-panel product y = H x for Q = 2 (plan in dq_panel.cpp): three or more subsystems whose last one has
+// 8 to 10 sites, and two such subsystems.
 //
 // Eq. (index) gives the last subsystem P_1 offset 0 and stride 1 inside the block of its particle
 // number, so the rows that share the pattern s0 of all other subsystems (the prefix P_0) form a
@@ -14,7 +15,8 @@
 //   - hops across the cut stage the partner panel s0 ^ bit_a in the warp's second slot;
 //   - inactive pairs read an element that holds zero, so the lanes never branch;
 //   - the row result (C + sum_k K_k n_k) X_i + sum_k A_k S_k is formed in 128-bit integers and
-//     rounded once, as in the two-subsystem panel kernel.
+//     rounded once, as in the panel kernel (the class sums S_k folded into two words for operators with
+//     more than 127 hops of one amplitude in a row).
 // No block barrier after the set-up: the warps of a CTA never wait for each other.
 #include <cstdint>
 

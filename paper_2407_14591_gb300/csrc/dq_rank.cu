@@ -6,9 +6,8 @@
 // local tables (16 bits an entry: a local pattern of at most 16 bits and its local index fit) once and takes
 // its share of the list, two states a thread and step.
 //
-// 2^24 states of 32 sites in three subsystems (35 KB of tables): unrank 262 -> 170 us, rank 410 -> 110 us
-//. Bound: integer
-// issue; the list itself, 16 bytes a state, takes 40 us of HBM time.
+// 2^24 states of 32 sites in three subsystems (35 KB of tables): unrank 262 -> 170 us, rank 410 -> 110 us.
+// Bound: integer issue; the list itself, 16 bytes a state, takes 40 us of HBM time.
 #include <cstdint>
 
 #include <cuda_runtime.h>
